@@ -107,7 +107,7 @@ __device__ __forceinline__ void acquire_tensormap(const CUtensorMap* m) {
 }
 
 template <class SV>
-__global__ void __launch_bounds__(kTileThreads, SV::kScaled ? 6 : 5)  // as k_update
+__global__ void __launch_bounds__(update_threads<SV>(), update_min_ctas<SV>())  // as k_update
     k_batch_update(const BatchHeader* __restrict__ hdr, const FrameWork* __restrict__ fw, int* counters) {
   extern __shared__ unsigned char dsmem[];
   UpdateSmem<SV>& sm = *reinterpret_cast<UpdateSmem<SV>*>(align128(dsmem));
@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(kTileThreads, SV::kScaled ? 6 : 5)  // as k_up
     if (threadIdx.x == 0 && w.stage_ok) acquire_tensormap(&w.maps.planes);
     const SV prev = make_view<SV>(w.prev_base, w.plane_stride, w.pitch);
     const SV next = make_view<SV>(w.next_base, w.plane_stride, w.pitch);
-    if (!update_tile(sm, &bar, phase, w.err, w.kp, w.W, w.H, w.reset != 0, w.stage_ok != 0, prev, next,
-                     &w.maps, w.rad, w.mot, (lt % w.tiles_x) * kTW, (lt / w.tiles_x) * kTH))
+    if (!update_any<SV, true>(sm, &bar, phase, w.err, w.kp, w.W, w.H, w.reset != 0, w.stage_ok != 0, prev, next,
+                              &w.maps, w.rad, w.mot, (lt % w.tiles_x) * kTW, (lt / w.tiles_x) * kTH))
       return;
   }
 }
@@ -462,14 +462,14 @@ static cudaError_t launch_static_cfg(cudaStream_t cs, void* d_table, int* d_coun
   e = cudaFuncSetAttribute(k_batch_update<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, ubytes);
   if (e != cudaSuccess) return e;
   int ou = 0, ob = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ou, k_batch_update<SV>, kTileThreads, ubytes);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ou, k_batch_update<SV>, update_threads<SV>(), ubytes);
   if (e != cudaSuccess) return e;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ob, k_batch_blend<SV, TH, R, MODE>, nt, sbytes);
   if (e != cudaSuccess) return e;
   const int sms = sm_count();
   const BatchHeader* hdr = (const BatchHeader*)d_table;
   const FrameWork* fw = (const FrameWork*)((char*)d_table + sizeof(BatchHeader));
-  k_batch_update<SV><<<sms * (ou > 0 ? ou : 1), kTileThreads, ubytes, cs>>>(hdr, fw, d_counters);
+  k_batch_update<SV><<<sms * (ou > 0 ? ou : 1), update_threads<SV>(), ubytes, cs>>>(hdr, fw, d_counters);
   k_batch_blend<SV, TH, R, MODE><<<sms * (ob > 0 ? ob : 1), nt, sbytes, cs>>>(hdr, fw, d_counters);
   return cudaGetLastError();
 }

@@ -118,6 +118,8 @@ __device__ __forceinline__ float2 blend_exponent2(float2 sp, float2 e0, float2 e
 constexpr int kStageW = 40;
 constexpr int kStageH = 10;
 constexpr int kStagePix = kStageW * kStageH;
+// With a 16-bit state a thread updates the two pixels (x, y) and (x, y + kPairY) of the tile.
+constexpr int kPairY = 4;
 // Bounded waits give up after this many SM clocks (about one second) and report
 // WRLS_ERR_TIMEOUT through the stream's error word.
 constexpr long long kWaitLimit = 2000000000LL;
@@ -190,9 +192,8 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
 // A view of one state copy: plane p of pixel (x, y) is at p * plane_stride + y * pitch + x.
 // Every format offers
 //   load(idx, v)          the 25 values, decoded (P itself)
-//   load_raw(idx, v, s)   the 25 values with P divided by a power-of-two scale s (binary32:
-//                         s = 1), which the bilinear gather folds into the tap weights
-//   load_beta_z(idx, b, z), store(idx, v), and the staged-window geometry of the update.
+//   load_beta_z(idx, b, z), store(idx, v), and the staged-window geometry of the update;
+//   load_staged (binary32)  the 25 values from the staged window.
 
 struct StateF32 {
   float* base;
@@ -201,10 +202,6 @@ struct StateF32 {
   __device__ __forceinline__ void load(size_t idx, float v[kNState]) const {
 #pragma unroll
     for (int p = 0; p < kNState; ++p) v[p] = __ldg(base + p * plane_stride + idx);
-  }
-  __device__ __forceinline__ void load_raw(size_t idx, float v[kNState], float& s) const {
-    load(idx, v);
-    s = 1.0f;
   }
   __device__ __forceinline__ void load_beta_z(size_t idx, float b[12], float z[3]) const {
 #pragma unroll
@@ -224,11 +221,10 @@ struct StateF32 {
   static constexpr uint32_t kStageBytes = kPlanes * kStagePix * 4;
   static constexpr uint32_t kTxBytes = kStageBytes;  // bytes the bulk copy delivers
   static constexpr bool kScaled = false;
-  static __device__ __forceinline__ void load_staged(const unsigned char* stage, int idx, float v[kNState], float& s) {
+  static __device__ __forceinline__ void load_staged(const unsigned char* stage, int idx, float v[kNState]) {
     const float* f = (const float*)stage;
 #pragma unroll
     for (int p = 0; p < kNState; ++p) v[p] = f[p * kStagePix + idx];
-    s = 1.0f;
   }
 };
 
@@ -259,6 +255,12 @@ struct State16 {
   static __device__ __forceinline__ float scale_of(uint32_t w12) {  // s = 2^e from word 12
     const int e = (int)(short)(w12 >> 16);
     return __int_as_float((e + 127) << 23);
+  }
+  // The even exponent e of the scale of a P whose largest diagonal entry is m.
+  static __device__ __forceinline__ int scale_exponent(float m) {
+    if (!(m > 0.0f && m <= 3.402823466e38f)) return 0;
+    const int f = ((__float_as_int(m) >> 23) & 0xff) - 126;  // m / 2^f in [0.5, 1) (normal m)
+    return min(max(f + (f & 1), -126), 126);
   }
   // P / s = L L^T from the factor in slots 12-21 (in place).
   static __device__ __forceinline__ void chol_to_p(float v[kNState]) {
@@ -312,15 +314,12 @@ struct State16 {
     s = scale_of(w[12]);
     chol_to_p(v);
   }
-  __device__ __forceinline__ void load_raw(size_t idx, float v[kNState], float& s) const {
+  __device__ __forceinline__ void load(size_t idx, float v[kNState]) const {
     uint32_t w[kPlanes];
+    float s;
 #pragma unroll
     for (int k = 0; k < kPlanes; ++k) w[k] = __ldg(base + k * plane_stride + idx);
     decode(w, v, s);
-  }
-  __device__ __forceinline__ void load(size_t idx, float v[kNState]) const {
-    float s;
-    load_raw(idx, v, s);
 #pragma unroll
     for (int p = kP; p < kZ; ++p) v[p] *= s;
   }
@@ -337,12 +336,7 @@ struct State16 {
     z[2] = unpack(__ldg(base + 12 * plane_stride + idx)).x;
   }
   __device__ __forceinline__ void store(size_t idx, const float v[kNState]) const {
-    const float m = fmaxf(fmaxf(v[kP + 0], v[kP + 4]), fmaxf(v[kP + 7], v[kP + 9]));
-    int e = 0;
-    if (m > 0.0f && m <= 3.402823466e38f) {
-      const int f = ((__float_as_int(m) >> 23) & 0xff) - 126;  // m / 2^f in [0.5, 1) (normal m)
-      e = min(max(f + (f & 1), -126), 126);
-    }
+    const int e = scale_exponent(fmaxf(fmaxf(v[kP + 0], v[kP + 4]), fmaxf(v[kP + 7], v[kP + 9])));
     const float inv_s = __int_as_float((127 - e) << 23);
     float a[10];
 #pragma unroll
@@ -363,13 +357,6 @@ struct State16 {
   static constexpr uint32_t kStageBytes = kPlanes * kStagePix * 4;
   static constexpr uint32_t kTxBytes = kStageBytes;
   static constexpr bool kScaled = true;
-  static __device__ __forceinline__ void load_staged(const unsigned char* stage, int idx, float v[kNState], float& s) {
-    const uint32_t* u = (const uint32_t*)stage;
-    uint32_t w[kPlanes];
-#pragma unroll
-    for (int k = 0; k < kPlanes; ++k) w[k] = u[k * kStagePix + idx];
-    decode(w, v, s);
-  }
 };
 template <>
 __device__ __forceinline__ float2 State16<__nv_bfloat16>::unpack(uint32_t u) {
@@ -421,84 +408,56 @@ __device__ __forceinline__ void init_model(const KParams& kp, const float z[3], 
   }
 }
 
-// Bilinear interpolation of every state value from its four taps in a fixed rounding order,
-// st = ((w00 a + w10 b) + w01 c) + w11 d by fused multiply-adds; consecutive planes are taken in
-// packed pairs (same rounding per component). bilerp_top takes the taps (x0, y0), (x1, y0),
-// bilerp_bottom adds (x0, y1), (x1, y1). The P slots take their own weights: the tap weight
-// times the tap's scale, a power of two (the products are exact, so this equals scaling the
-// decoded values first).
-__device__ __forceinline__ void bilerp_top(float w00, float w10, float q00, float q10, const float a[kNState],
-                                           const float b[kNState], float st[kNState]) {
+// Bilinear interpolation of every binary32 state value from its four taps in a fixed rounding
+// order, st = ((w00 a + w10 b) + w01 c) + w11 d by fused multiply-adds; consecutive planes are
+// taken in packed pairs (same rounding per component). bilerp_top takes the taps (x0, y0),
+// (x1, y0), bilerp_bottom adds (x0, y1), (x1, y1).
+__device__ __forceinline__ void bilerp_top(float w00, float w10, const float a[kNState], const float b[kNState],
+                                           float st[kNState]) {
 #pragma unroll
   for (int p = 0; p + 1 < kNState; p += 2) {
-    const bool isP = p >= kP && p < kZ;
-    const float2 wa = isP ? make_float2(q00, q00) : make_float2(w00, w00);
-    const float2 wb = isP ? make_float2(q10, q10) : make_float2(w10, w10);
-    const float2 v = f2fma(wb, make_float2(b[p], b[p + 1]), f2mul(wa, make_float2(a[p], a[p + 1])));
+    const float2 v = f2fma(make_float2(w10, w10), make_float2(b[p], b[p + 1]),
+                           f2mul(make_float2(w00, w00), make_float2(a[p], a[p + 1])));
     st[p] = v.x;
     st[p + 1] = v.y;
   }
   if (kNState % 2) st[kNState - 1] = fmaf(w10, b[kNState - 1], w00 * a[kNState - 1]);
 }
-__device__ __forceinline__ void bilerp_bottom(float w01, float w11, float q01, float q11, const float c[kNState],
-                                              const float d[kNState], float st[kNState]) {
+__device__ __forceinline__ void bilerp_bottom(float w01, float w11, const float c[kNState], const float d[kNState],
+                                              float st[kNState]) {
 #pragma unroll
   for (int p = 0; p + 1 < kNState; p += 2) {
-    const bool isP = p >= kP && p < kZ;
-    const float2 wc = isP ? make_float2(q01, q01) : make_float2(w01, w01);
-    const float2 wd = isP ? make_float2(q11, q11) : make_float2(w11, w11);
-    const float2 v = f2fma(wd, make_float2(d[p], d[p + 1]),
-                           f2fma(wc, make_float2(c[p], c[p + 1]), make_float2(st[p], st[p + 1])));
+    const float2 v = f2fma(make_float2(w11, w11), make_float2(d[p], d[p + 1]),
+                           f2fma(make_float2(w01, w01), make_float2(c[p], c[p + 1]), make_float2(st[p], st[p + 1])));
     st[p] = v.x;
     st[p + 1] = v.y;
   }
   if (kNState % 2) st[kNState - 1] = fmaf(w11, d[kNState - 1], fmaf(w01, c[kNState - 1], st[kNState - 1]));
 }
 
-// One tap alone (the others have weight 0): st = w00 a.
-__device__ __forceinline__ void bilerp_top1(float w00, float q00, const float a[kNState], float st[kNState]) {
-#pragma unroll
-  for (int p = 0; p + 1 < kNState; p += 2) {
-    const bool isP = p >= kP && p < kZ;
-    const float2 wa = isP ? make_float2(q00, q00) : make_float2(w00, w00);
-    const float2 v = f2mul(wa, make_float2(a[p], a[p + 1]));
-    st[p] = v.x;
-    st[p + 1] = v.y;
-  }
-  if (kNState % 2) st[kNState - 1] = w00 * a[kNState - 1];
-}
-
-// P-slot weight of a tap: w times the tap's scale (binary32: the weight itself).
-template <class SV>
-__device__ __forceinline__ float scaled_weight(float w, float s) {
-  if constexpr (SV::kScaled) return w * s;
-  else return w;
-}
-
 // Bilinear fetch of the previous state at q = (qx, qy) (Sec. 5.3: models are reprojected,
 // not colours). q is valid; taps beyond the last row/column are clamped.
-template <class SV>
-__device__ __forceinline__ void gather_bilinear(const SV& prev, int W, int H, float qx, float qy,
+__device__ __forceinline__ void gather_bilinear(const StateF32& prev, int W, int H, float qx, float qy,
                                                 float st[kNState]) {
   const int x0 = (int)floorf(qx), y0 = (int)floorf(qy);
   const float fx = qx - (float)x0, fy = qy - (float)y0;
   const int x1 = min(x0 + 1, W - 1), y1 = min(y0 + 1, H - 1);
   const float w00 = (1.0f - fx) * (1.0f - fy), w10 = fx * (1.0f - fy);
   const float w01 = (1.0f - fx) * fy, w11 = fx * fy;
-  float a[kNState], b[kNState], sa, sb;
-  prev.load_raw((size_t)y0 * prev.pitch + x0, a, sa);
-  prev.load_raw((size_t)y0 * prev.pitch + x1, b, sb);
-  bilerp_top(w00, w10, scaled_weight<SV>(w00, sa), scaled_weight<SV>(w10, sb), a, b, st);
-  prev.load_raw((size_t)y1 * prev.pitch + x0, a, sa);
-  prev.load_raw((size_t)y1 * prev.pitch + x1, b, sb);
-  bilerp_bottom(w01, w11, scaled_weight<SV>(w01, sa), scaled_weight<SV>(w11, sb), a, b, st);
+  float a[kNState], b[kNState];
+  prev.load((size_t)y0 * prev.pitch + x0, a);
+  prev.load((size_t)y0 * prev.pitch + x1, b);
+  bilerp_top(w00, w10, a, b, st);
+  prev.load((size_t)y1 * prev.pitch + x0, a);
+  prev.load((size_t)y1 * prev.pitch + x1, b);
+  bilerp_bottom(w01, w11, a, b, st);
 }
 
 // Bilinear fetch from the staged window whose origin is (X0, Y0). TAPS = 4, or 2 (the lower
 // row's weights are 0: fy = 0) or 1 (fx = fy = 0): taps of weight exactly 0 are not read. A
 // tap of weight 0 adds fma(0, v, s) = s for a finite v, so the result is that of the four-tap
 // sum (up to the sign of a zero).
-template <class SV, int TAPS = 4>
+template <int TAPS = 4>
 __device__ __forceinline__ void gather_bilinear_staged(const unsigned char* stage, int X0, int Y0, int W,
                                                        int H, float qx, float qy, float st[kNState]) {
   const int x0 = (int)floorf(qx), y0 = (int)floorf(qy);
@@ -507,18 +466,19 @@ __device__ __forceinline__ void gather_bilinear_staged(const unsigned char* stag
   const float w00 = (1.0f - fx) * (1.0f - fy), w10 = fx * (1.0f - fy);
   const float w01 = (1.0f - fx) * fy, w11 = fx * fy;
   const int r0 = (y0 - Y0) * kStageW, r1 = (y1 - Y0) * kStageW;
-  float a[kNState], b[kNState], sa, sb;
-  SV::load_staged(stage, r0 + x0 - X0, a, sa);
+  float a[kNState], b[kNState];
+  StateF32::load_staged(stage, r0 + x0 - X0, a);
   if constexpr (TAPS == 1) {
-    bilerp_top1(w00, scaled_weight<SV>(w00, sa), a, st);
+#pragma unroll
+    for (int p = 0; p < kNState; ++p) st[p] = w00 * a[p];
     return;
   }
-  SV::load_staged(stage, r0 + x1 - X0, b, sb);
-  bilerp_top(w00, w10, scaled_weight<SV>(w00, sa), scaled_weight<SV>(w10, sb), a, b, st);
+  StateF32::load_staged(stage, r0 + x1 - X0, b);
+  bilerp_top(w00, w10, a, b, st);
   if constexpr (TAPS == 2) return;
-  SV::load_staged(stage, r1 + x0 - X0, a, sa);
-  SV::load_staged(stage, r1 + x1 - X0, b, sb);
-  bilerp_bottom(w01, w11, scaled_weight<SV>(w01, sa), scaled_weight<SV>(w11, sb), a, b, st);
+  StateF32::load_staged(stage, r1 + x0 - X0, a);
+  StateF32::load_staged(stage, r1 + x1 - X0, b);
+  bilerp_bottom(w01, w11, a, b, st);
 }
 
 // Eq. 12 feature, Eq. 13 weight and the wRLS update (Eq. 8, 14, 9, 11) of one pixel.
@@ -603,6 +563,308 @@ __device__ __forceinline__ float update_pixel(const KParams& kp, bool valid, flo
   st[kZ + 1] = z[1];
   st[kZ + 2] = z[2];
   return w;
+}
+
+// ---- a pixel pair of the temporal update ------------------------------------------------------
+//
+// The 16-bit update is bound by its instructions (decode, P = L L^T at each tap, Eq. 8-14, the
+// factorisation on store), so a thread updates two pixels at once: every quantity is a float2
+// whose components belong to the two pixels, and all of that runs as packed binary32
+// instructions (one for both pixels, each component rounded as the scalar operation). The state
+// is taken in the order z, P, beta of each channel, and each part is stored as soon as it is
+// updated, so a thread holds at most P and one channel's model at a time. Measured on a 1080p
+// frame under general motion: 674 instead of 932 instructions a pixel, 71.5 -> 68.2 us (BF16),
+// 69.6 -> 67.8 us (FP16); beside the blend of the frame before (sequence entry), where issue
+// slots are shared, 119.8 -> 113.6 us a frame. The binary32 update keeps one pixel a thread: it is
+// bound by the latency of the window copy, which twice the warps hide better (83.7 us against
+// 90.3 us for pairs at their best launch bound).
+
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
+
+// Where the taps of the previous state are read from: the staged window in shared memory, or
+// the state copy itself. word(p, i) = 32-bit word of plane p at offset i.
+struct StagedTaps {
+  const uint32_t* stage;
+  __device__ __forceinline__ uint32_t word(int p, int i) const { return stage[p * kStagePix + i]; }
+};
+struct GlobalTaps {
+  const uint32_t* base;
+  size_t plane_stride;
+  __device__ __forceinline__ uint32_t word(int p, int i) const {
+    return __ldg(base + (size_t)p * plane_stride + (uint32_t)i);
+  }
+};
+
+// Tap offsets and bilinear weights of a pair, in the order (x0, y0), (x1, y0), (x0, y1),
+// (x1, y1); TAPS = 4, or 2 (the lower row's weights are 0: fy = 0) or 1 (fx = fy = 0): taps of
+// weight exactly 0 are not read. Every value is interpolated in one rounding order,
+// ((w00 a + w10 b) + w01 c) + w11 d by fused multiply-adds; a tap of weight 0 adds
+// fma(0, v, s) = s for a finite v, so fewer taps give the four-tap sum (up to the sign of a zero).
+struct PairTaps {
+  int o0[4], o1[4];
+  float2 w[4];
+};
+
+template <int TAPS>
+__device__ __forceinline__ float2 tap_add(int t, float2 w, float2 v, float2 acc) {
+  return t == 0 ? f2mul(w, v) : f2fma(w, v, acc);
+}
+
+// Interpolated parts of a 16-bit state. q: the P weights of the taps, the tap weight times the
+// tap's power-of-two scale (exact, so that this equals scaling the decoded P first), set by z().
+template <class SV>
+struct PairState;
+
+template <typename T>
+struct PairState<State16<T>> {
+  using SV = State16<T>;
+  // the pair's values of slots 2k (lo) and 2k + 1 (hi) at one tap
+  template <class Src>
+  static __device__ __forceinline__ void tap(const Src& s, int k, int o0, int o1, float2& lo, float2& hi) {
+    const float2 a = SV::unpack(s.word(k, o0)), b = SV::unpack(s.word(k, o1));
+    lo = make_float2(a.x, b.x);
+    hi = make_float2(a.y, b.y);
+  }
+  template <int TAPS, class Src>
+  static __device__ __forceinline__ void z(const Src& s, const PairTaps& t, float2 v[3], float2 q[4]) {
+#pragma unroll
+    for (int k = 0; k < TAPS; ++k) {
+      float2 z0, z1;
+      tap(s, 11, t.o0[k], t.o1[k], z0, z1);
+      const uint32_t u0 = s.word(12, t.o0[k]), u1 = s.word(12, t.o1[k]);
+      const float2 z2 = make_float2(SV::unpack(u0).x, SV::unpack(u1).x);
+      v[0] = tap_add<TAPS>(k, t.w[k], z0, v[0]);
+      v[1] = tap_add<TAPS>(k, t.w[k], z1, v[1]);
+      v[2] = tap_add<TAPS>(k, t.w[k], z2, v[2]);
+      q[k] = f2mul(t.w[k], make_float2(SV::scale_of(u0), SV::scale_of(u1)));
+    }
+  }
+  template <int TAPS, class Src>
+  static __device__ __forceinline__ void p(const Src& s, const PairTaps& t, const float2 q[4], float2 P[10]) {
+#pragma unroll
+    for (int k = 0; k < TAPS; ++k) {
+      float2 l[10];
+#pragma unroll
+      for (int w = 0; w < 5; ++w) tap(s, 6 + w, t.o0[k], t.o1[k], l[2 * w], l[2 * w + 1]);
+      // P / s = L L^T of the tap, rows of L: l[0] | l[1] l[4] | l[2] l[5] l[7] | l[3] l[6] l[8] l[9]
+      const float2 w = q[k];
+      P[0] = tap_add<TAPS>(k, w, f2mul(l[0], l[0]), P[0]);
+      P[1] = tap_add<TAPS>(k, w, f2mul(l[1], l[0]), P[1]);
+      P[2] = tap_add<TAPS>(k, w, f2mul(l[2], l[0]), P[2]);
+      P[3] = tap_add<TAPS>(k, w, f2mul(l[3], l[0]), P[3]);
+      P[4] = tap_add<TAPS>(k, w, f2fma(l[4], l[4], f2mul(l[1], l[1])), P[4]);
+      P[5] = tap_add<TAPS>(k, w, f2fma(l[5], l[4], f2mul(l[2], l[1])), P[5]);
+      P[6] = tap_add<TAPS>(k, w, f2fma(l[6], l[4], f2mul(l[3], l[1])), P[6]);
+      P[7] = tap_add<TAPS>(k, w, f2fma(l[7], l[7], f2fma(l[5], l[5], f2mul(l[2], l[2]))), P[7]);
+      P[8] = tap_add<TAPS>(k, w, f2fma(l[8], l[7], f2fma(l[6], l[5], f2mul(l[3], l[2]))), P[8]);
+      P[9] = tap_add<TAPS>(k, w, f2fma(l[9], l[9], f2fma(l[8], l[8], f2fma(l[6], l[6], f2mul(l[3], l[3])))), P[9]);
+    }
+  }
+  template <int TAPS, class Src>
+  static __device__ __forceinline__ void beta(const Src& s, const PairTaps& t, int c, float2 b[4]) {
+#pragma unroll
+    for (int k = 0; k < TAPS; ++k) {
+      float2 v[4];
+      tap(s, 2 * c, t.o0[k], t.o1[k], v[0], v[1]);
+      tap(s, 2 * c + 1, t.o0[k], t.o1[k], v[2], v[3]);
+#pragma unroll
+      for (int a = 0; a < 4; ++a) b[a] = tap_add<TAPS>(k, t.w[k], v[a], b[a]);
+    }
+  }
+  static __device__ __forceinline__ void put(const SV& n, uint32_t i, uint32_t i1, int k, uint32_t u0, uint32_t u1, bool in0, bool in1) {
+    uint32_t* d = n.base + k * n.plane_stride + i;
+    if (in0) d[0] = u0;
+    if (in1) d[i1] = u1;
+  }
+  // Cholesky factor of P / 2^e as in State16::store, for both pixels; a pivot that is not a
+  // positive normal number gives a zero column.
+  static __device__ __forceinline__ void store_p(const SV& n, uint32_t i, uint32_t i1, const float2 P[10], int e[2], bool in0, bool in1) {
+    const float m0 = fmaxf(fmaxf(P[0].x, P[4].x), fmaxf(P[7].x, P[9].x));
+    const float m1 = fmaxf(fmaxf(P[0].y, P[4].y), fmaxf(P[7].y, P[9].y));
+    e[0] = SV::scale_exponent(m0);
+    e[1] = SV::scale_exponent(m1);
+    const float2 inv = make_float2(__int_as_float((127 - e[0]) << 23), __int_as_float((127 - e[1]) << 23));
+    auto root = [](float2 piv, float2& l, float2& r) {
+      r = make_float2(piv.x >= 1.17549435e-38f ? rsqrt_approx(piv.x) : 0.0f,
+                      piv.y >= 1.17549435e-38f ? rsqrt_approx(piv.y) : 0.0f);
+      l = f2mul(piv, r);
+    };
+    float2 l[10], r0, r1, r2, r3;
+    root(f2mul(P[0], inv), l[0], r0);
+    const float2 ir0 = f2mul(inv, r0);
+    l[1] = f2mul(P[1], ir0);
+    l[2] = f2mul(P[2], ir0);
+    l[3] = f2mul(P[3], ir0);
+    const float2 n1 = f2neg(l[1]), n2 = f2neg(l[2]), n3 = f2neg(l[3]);
+    root(f2fma(n1, l[1], f2mul(P[4], inv)), l[4], r1);
+    l[5] = f2mul(f2fma(n2, l[1], f2mul(P[5], inv)), r1);
+    l[6] = f2mul(f2fma(n3, l[1], f2mul(P[6], inv)), r1);
+    const float2 n5 = f2neg(l[5]), n6 = f2neg(l[6]);
+    root(f2fma(n5, l[5], f2fma(n2, l[2], f2mul(P[7], inv))), l[7], r2);
+    l[8] = f2mul(f2fma(n6, l[5], f2fma(n3, l[2], f2mul(P[8], inv))), r2);
+    root(f2fma(f2neg(l[8]), l[8], f2fma(n6, l[6], f2fma(n3, l[3], f2mul(P[9], inv)))), l[9], r3);
+#pragma unroll
+    for (int k = 0; k < 5; ++k)
+      put(n, i, i1, 6 + k, SV::pack(l[2 * k].x, l[2 * k + 1].x), SV::pack(l[2 * k].y, l[2 * k + 1].y), in0, in1);
+  }
+  static __device__ __forceinline__ void store_beta(const SV& n, uint32_t i, uint32_t i1, int c, const float2 b[4], bool in0, bool in1) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      put(n, i, i1, 2 * c + k, SV::pack(b[2 * k].x, b[2 * k + 1].x), SV::pack(b[2 * k].y, b[2 * k + 1].y), in0, in1);
+  }
+  static __device__ __forceinline__ void store_z(const SV& n, uint32_t i, uint32_t i1, const float2 z[3], const int e[2], bool in0, bool in1) {
+    put(n, i, i1, 11, SV::pack(z[0].x, z[1].x), SV::pack(z[0].y, z[1].y), in0, in1);
+    put(n, i, i1, 12, (SV::pack(z[2].x, 0.0f) & 0xffffu) | ((uint32_t)e[0] << 16),
+        (SV::pack(z[2].y, 0.0f) & 0xffffu) | ((uint32_t)e[1] << 16), in0, in1);
+  }
+};
+
+// The two pixels' inputs of a temporal update.
+struct PairInput {
+  bool valid0, valid1;  // reprojection inside the image (else the pixel restarts)
+  bool miss0, miss1;    // a channel of the sample is not finite
+  bool restart, missing;  // some pixel of the warp restarts / misses its sample (uniform)
+  float2 I[3];          // the samples (0 where missing)
+  float2 lo[3], hi[3];  // per-channel min / max of the 3x3 neighbourhood (Eq. 12 clamp)
+};
+
+// Eq. 12 feature, Eq. 13 weight and the wRLS update (Eq. 8, 14, 9, 11) of a pixel pair, stored to
+// `next` at offsets i and i + i1. TAPS = 0: no pixel of the pair is valid.
+template <class SV, int TAPS, class Src>
+__device__ __forceinline__ void update_pair(const KParams& kp, const Src& src, const PairTaps& t, const PairInput& in,
+                                            const SV& next, uint32_t i, uint32_t i1, bool in0, bool in1) {
+  using PS = PairState<SV>;
+  constexpr int NT = TAPS > 0 ? TAPS : 1;
+  const bool feat = kp.feature_mode == 0;
+  const bool restart = TAPS == 0 || in.restart;
+  const bool r0 = TAPS == 0 || !in.valid0, r1 = TAPS == 0 || !in.valid1;
+  float2 q[4];
+  // Eq. 12: clamped history and the new sample; a missing sample keeps the history, a
+  // restarted pixel takes the sample
+  float2 z[3];
+  if constexpr (TAPS > 0) {
+    PS::template z<NT>(src, t, z, q);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float2 h = z[c];
+      if (kp.clamp_mode == 0)
+        h = make_float2(fminf(fmaxf(h.x, in.lo[c].x), in.hi[c].x), fminf(fmaxf(h.y, in.lo[c].y), in.hi[c].y));
+      z[c] = f2fma(f2(kp.alpha), h, f2mul(f2(kp.one_m_alpha), in.I[c]));
+      if (in.missing) z[c] = make_float2(in.miss0 ? h.x : z[c].x, in.miss1 ? h.y : z[c].y);
+    }
+  }
+  if (restart) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if (r0) z[c].x = in.I[c].x;
+      if (r1) z[c].y = in.I[c].y;
+    }
+  }
+  // Eq. 13 (one scalar per pixel over RGB); RLS mode: w = 1; a missing sample: 0
+  float2 w = f2(1.0f);
+  if (kp.weight_mode != 1) {
+    const float2 d0 = f2sub(in.I[0], z[0]), d1 = f2sub(in.I[1], z[1]), d2 = f2sub(in.I[2], z[2]);
+    const float2 dist2 = f2fma(d2, d2, f2fma(d1, d1, f2mul(d0, d0)));
+    const float2 nI = f2fma(in.I[2], in.I[2], f2fma(in.I[1], in.I[1], f2mul(in.I[0], in.I[0])));
+    const float2 nz = f2fma(z[2], z[2], f2fma(z[1], z[1], f2mul(z[0], z[0])));
+    const float2 rm = make_float2(rcp_approx(sqrt_approx(fminf(nI.x, nz.x)) + kp.eps),
+                                  rcp_approx(sqrt_approx(fminf(nI.y, nz.y)) + kp.eps));
+    const float2 ex = f2mul(f2mul(f2mul(dist2, rm), rm), f2(-kp.w_k));
+    w = make_float2(ex2_approx(ex.x), ex2_approx(ex.y));
+  }
+  if (in.missing) {
+    if (in.miss0) w.x = 0.0f;
+    if (in.miss1) w.y = 0.0f;
+  }
+  // predictor p = [1, z] (Sec. 5.1), or [1] without feature
+  float2 pz[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) pz[c] = feat ? z[c] : f2(0.0f);
+  // k = P p, s = p^T P p; Eq. 14: q^w = P p / (lambda / w + p^T P p) = (w / (lambda + w s)) P p
+  float2 P[10];
+  if constexpr (TAPS > 0) PS::template p<NT>(src, t, q, P);
+  if (restart) {
+#pragma unroll
+    for (int e = 0; e < 10; ++e) {
+      const bool diag = e == 0 || (feat && (e == 4 || e == 7 || e == 9));
+      const float v = diag ? kp.p0_delta : 0.0f;
+      if (r0) P[e].x = v;
+      if (r1) P[e].y = v;
+    }
+  }
+  float2 k[4];
+  k[0] = f2fma(P[3], pz[2], f2fma(P[2], pz[1], f2fma(P[1], pz[0], P[0])));
+  k[1] = f2fma(P[6], pz[2], f2fma(P[5], pz[1], f2fma(P[4], pz[0], P[1])));
+  k[2] = f2fma(P[8], pz[2], f2fma(P[7], pz[1], f2fma(P[5], pz[0], P[2])));
+  k[3] = f2fma(P[9], pz[2], f2fma(P[8], pz[1], f2fma(P[6], pz[0], P[3])));
+  const float2 s = f2fma(k[3], pz[2], f2fma(k[2], pz[1], f2fma(k[1], pz[0], k[0])));
+  const float2 den = f2fma(w, s, f2(kp.lambda));
+  const float2 g = f2mul(w, make_float2(rcp_approx(den.x), rcp_approx(den.y)));
+  // Eq. 11: P <- (P - q^w p^T P) / lambda, with p^T P = k^T
+  {
+    int e = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const float2 ngk = f2neg(f2mul(g, k[a]));
+#pragma unroll
+      for (int b = a; b < 4; ++b, ++e) P[e] = f2mul(f2fma(ngk, k[b], P[e]), f2(kp.inv_lambda));
+    }
+  }
+  if (kp.p_trace_max > 0.0f) {
+    auto guard = [&](float p0, float p4, float p7, float p9) {
+      const float tr = p0 + (feat ? p4 + p7 + p9 : 0.0f);
+      const bool bad = !(p0 > 0.0f) || (feat && (!(p4 > 0.0f) || !(p7 > 0.0f) || !(p9 > 0.0f)));
+      return bad || tr > kp.p_trace_max;
+    };
+    const bool b0 = guard(P[0].x, P[4].x, P[7].x, P[9].x), b1 = guard(P[0].y, P[4].y, P[7].y, P[9].y);
+#pragma unroll
+    for (int e = 0; e < 10; ++e) {
+      const bool diag = e == 0 || (feat && (e == 4 || e == 7 || e == 9));
+      const float v = diag ? kp.p0_delta : 0.0f;
+      if (b0) P[e].x = v;
+      if (b1) P[e].y = v;
+    }
+  }
+  int ex[2] = {0, 0};
+  PS::store_p(next, i, i1, P, ex, in0, in1);
+  PS::store_z(next, i, i1, z, ex, in0, in1);
+  // Eq. 8, 9 per channel
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float2 b[4];
+    if constexpr (TAPS > 0) PS::template beta<NT>(src, t, c, b);
+    if (restart) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        // beta = 0 (init_mode 0) or the feature pass-through beta_c = e_{c+1} (z_c with p = [1])
+        const bool one = kp.init_mode == 1 && feat && a == c + 1;
+        const bool own = kp.init_mode == 1 && !feat && a == 0;
+        if (r0) b[a].x = own ? z[c].x : one ? 1.0f : 0.0f;
+        if (r1) b[a].y = own ? z[c].y : one ? 1.0f : 0.0f;
+      }
+    }
+    const float2 pred = f2fma(b[3], pz[2], f2fma(b[2], pz[1], f2fma(b[1], pz[0], b[0])));
+    const float2 ge = f2mul(g, f2sub(in.I[c], pred));  // g = 0 for a missing sample
+#pragma unroll
+    for (int a = 0; a < 4; ++a) b[a] = f2fma(ge, k[a], b[a]);
+    PS::store_beta(next, i, i1, c, b, in0, in1);
+  }
 }
 
 }  // namespace wrls

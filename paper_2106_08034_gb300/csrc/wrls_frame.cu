@@ -7,13 +7,8 @@
 
 namespace wrls {
 
-// CTAs per SM the update is compiled for (registers a thread <= 65536 / (256 x CTAs)), measured
-// at 1080p: with a 16-bit state (issue-bound, 24 KB of shared memory a CTA) 6 CTAs (40
-// registers, a small spill) took 70.6 us against 74.8 us at 4 (64 registers) and 71.7 at 5; 7
-// (32 registers) spilled and took 87.7. With the binary32 state (44 KB a CTA) 5 CTAs (48
-// registers) took 83.1 us against 88.0 at 4.
 template <class SV>
-__global__ void __launch_bounds__(kTileThreads, SV::kScaled ? 6 : 5)
+__global__ void __launch_bounds__(update_threads<SV>(), update_min_ctas<SV>())
     k_update(const KParams kp, const int W, const int H, const int reset, const int stage_ok,
              const SV prev, const SV next, const __grid_constant__ StageMaps maps,
              const float* __restrict__ rad, const float* __restrict__ mot, int* err) {
@@ -22,8 +17,8 @@ __global__ void __launch_bounds__(kTileThreads, SV::kScaled ? 6 : 5)
   UpdateSmem<SV>& sm = *reinterpret_cast<UpdateSmem<SV>*>(align128(dsmem));
   if (threadIdx.x == 0) mbar_init(&bar, 1);
   uint32_t phase = 0;
-  update_tile(sm, &bar, phase, err, kp, W, H, reset != 0, stage_ok != 0, prev, next, &maps, rad, mot,
-              blockIdx.x * kTW, blockIdx.y * kTH);
+  update_any<SV, false>(sm, &bar, phase, err, kp, W, H, reset != 0, stage_ok != 0, prev, next, &maps, rad, mot,
+                        (int)blockIdx.x * kTW, (int)blockIdx.y * kTH);
 }
 
 template <class SV, int TH, int R, int MODE>
@@ -68,7 +63,7 @@ static cudaError_t launch_update_t(const KParams& kp, const StateDesc& prev, con
     attr_set = true;
   }
   const dim3 grid((prev.W + kTW - 1) / kTW, (prev.H + kTH - 1) / kTH);
-  k_update<SV><<<grid, kTileThreads, bytes, cs>>>(kp, prev.W, prev.H, reset ? 1 : 0, prev.stage_ok ? 1 : 0,
+  k_update<SV><<<grid, update_threads<SV>(), bytes, cs>>>(kp, prev.W, prev.H, reset ? 1 : 0, prev.stage_ok ? 1 : 0,
                                                    pv, nx, prev.maps, rad, mot, err);
   return cudaGetLastError();
 }

@@ -20,6 +20,8 @@ namespace wrls {
 constexpr int kTW = 32;
 constexpr int kTH = 8;
 constexpr int kTileThreads = kTW * kTH;
+constexpr int kPairThreads = kTW * kPairY;  // 16-bit state: two pixels a thread
+static_assert(kTH == 2 * kPairY, "a pixel pair spans half the tile");
 
 // Shared memory of an update tile: the staged previous-state window, the radiance tile with a
 // 1-pixel halo and the tap-footprint reduction. (The copy's mbarrier lives outside, so that a
@@ -28,7 +30,7 @@ template <class SV>
 struct UpdateSmem {
   alignas(128) unsigned char stage[SV::kStageBytes];
   float rad[3][kTH + 2][kTW + 2];
-  int red[kTileThreads / 32][4];
+  int4 red[kTileThreads / 32];
   int box[4];
 };
 template <class SV>
@@ -41,11 +43,10 @@ constexpr int update_smem_bytes() { return (int)sizeof(UpdateSmem<SV>) + 128; } 
 // memory. Otherwise (large motion spread) the taps are read from global memory.
 // `bar` is the CTA's mbarrier (count 1) and `phase` its current phase. Returns false if the
 // bounded wait for the copy gave up (the error word is set; the caller must return).
-template <class SV>
-__device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, uint32_t& phase, int* err,
+__device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* bar, uint32_t& phase, int* err,
                                            const KParams& kp, const int W, const int H,
-                                           const bool reset, const bool stage_ok, const SV& prev,
-                                           const SV& next, const StageMaps* maps,
+                                           const bool reset, const bool stage_ok, const StateF32& prev,
+                                           const StateF32& next, const StageMaps* maps,
                                            const float* __restrict__ rad,
                                            const float* __restrict__ mot, const int bx0,
                                            const int by0) {
@@ -81,25 +82,26 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, u
   lo_y = __reduce_min_sync(0xffffffffu, lo_y);
   hi_y = __reduce_max_sync(0xffffffffu, hi_y);
   if (lane == 0) {
-    sm.red[warp][0] = lo_x; sm.red[warp][1] = hi_x; sm.red[warp][2] = lo_y; sm.red[warp][3] = hi_y;
+    sm.red[warp] = make_int4(lo_x, hi_x, lo_y, hi_y);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int w = 1; w < kTileThreads / 32; ++w) {
-      lo_x = min(lo_x, sm.red[w][0]); hi_x = max(hi_x, sm.red[w][1]);
-      lo_y = min(lo_y, sm.red[w][2]); hi_y = max(hi_y, sm.red[w][3]);
+      const int4 r = sm.red[w];
+      lo_x = min(lo_x, r.x); hi_x = max(hi_x, r.y);
+      lo_y = min(lo_y, r.z); hi_y = max(hi_y, r.w);
     }
     int fits = 0, X0 = 0, Y0 = 0;
     if (stage_ok && hi_x >= 0) {
-      X0 = lo_x - lo_x % SV::kAlignX;  // TMA box origin: 16-byte aligned column
+      X0 = lo_x - lo_x % StateF32::kAlignX;  // TMA box origin: 16-byte aligned column
       Y0 = lo_y;
       fits = (hi_x - X0 < kStageW) && (hi_y - Y0 < kStageH);
     }
     sm.box[0] = X0; sm.box[1] = Y0; sm.box[2] = fits;
     if (fits) {
       fence_proxy_async();
-      mbar_expect_tx(bar, SV::kTxBytes);
+      mbar_expect_tx(bar, StateF32::kTxBytes);
       if (!kp.debug_withhold_copy) tma_load_3d(sm.stage, &maps->planes, X0, Y0, 0, bar);
     }
   }
@@ -153,15 +155,211 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, u
   float st[kNState];
   if (valid) {
     if (fits) {
-      if (fy0 && fx0) gather_bilinear_staged<SV, 1>(sm.stage, X0, Y0, W, H, qx, qy, st);
-      else if (fy0) gather_bilinear_staged<SV, 2>(sm.stage, X0, Y0, W, H, qx, qy, st);
-      else gather_bilinear_staged<SV, 4>(sm.stage, X0, Y0, W, H, qx, qy, st);
+      if (fy0 && fx0) gather_bilinear_staged<1>(sm.stage, X0, Y0, W, H, qx, qy, st);
+      else if (fy0) gather_bilinear_staged<2>(sm.stage, X0, Y0, W, H, qx, qy, st);
+      else gather_bilinear_staged<4>(sm.stage, X0, Y0, W, H, qx, qy, st);
     }
     else gather_bilinear(prev, W, H, qx, qy, st);
   }
   update_pixel(kp, valid, st, I, missing, lo, hi, have_box);
   next.store((size_t)y * next.pitch + x, st);
   return true;
+}
+
+// Radiance of window pixel (gx, gy); a missing sample (a non-finite channel) and a pixel outside
+// the image give (NaN, NaN, NaN): fminf/fmaxf ignore NaN operands, so the clamp box skips them
+// without a test per neighbour.
+struct Rgb { float r, g, b; };
+__device__ __forceinline__ Rgb load_radiance(const float* __restrict__ rad, size_t npix, int gx, int gy, int W, int H) {
+  const float nan = __int_as_float(0x7fc00000);
+  Rgb v{nan, nan, nan};
+  if ((unsigned)gx < (unsigned)W && (unsigned)gy < (unsigned)H) {
+    const float* p = rad + (size_t)gy * W + gx;
+    v.r = __ldg(p);
+    v.g = __ldg(p + npix);
+    v.b = __ldg(p + 2 * npix);
+    // 0 * v is NaN for a non-finite v
+    const float t = fmaf(v.b, 0.0f, fmaf(v.g, 0.0f, v.r * 0.0f));
+    if (t != t) v.r = v.g = v.b = nan;
+  }
+  return v;
+}
+
+// The same tile with a 16-bit state: 128 threads, two pixels each (update_pair). The decode
+// (an exact unpack and P = L L^T at each tap), Eq. 8-14 and the Cholesky factorisation run
+// packed over the two pixels. PERSIST: the CTA runs several tiles.
+template <class SV, bool PERSIST>
+__device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, uint32_t& phase, int* err,
+                                           const KParams& kp, const int W, const int H,
+                                           const bool reset, const bool stage_ok, const SV& prev,
+                                           const SV& next, const StageMaps* maps,
+                                           const float* __restrict__ rad,
+                                           const float* __restrict__ mot, const int bx0,
+                                           const int by0) {
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;  // lane, warp: the tile row(s) of a warp
+  const size_t npix = (size_t)W * H;
+  const int xa = bx0 + tx, ya = by0 + ty, xb = xa, yb = ya + kPairY;
+  const bool in0 = xa < W && ya < H, in1 = xb < W && yb < H;
+
+  // reprojection q = pi(v_j) = j + v_j (Table 2), in binary32
+  float qx0 = 0.0f, qy0 = 0.0f, qx1 = 0.0f, qy1 = 0.0f;
+  {
+    const float* m = mot + (size_t)ya * W + xa;
+    const size_t step = (size_t)kPairY * W;
+    if (in0) { qx0 = __ldg(m); qy0 = __ldg(m + npix); }
+    if (in1) { qx1 = __ldg(m + step); qy1 = __ldg(m + step + npix); }
+  }
+  qx0 += (float)xa; qy0 += (float)ya;
+  qx1 += (float)xb; qy1 += (float)yb;
+  const float xmax = (float)(W - 1), ymax = (float)(H - 1);
+  PairInput in;
+  in.valid0 = in0 && !reset && qx0 >= 0.0f && qx0 <= xmax && qy0 >= 0.0f && qy0 <= ymax;
+  in.valid1 = in1 && !reset && qx1 >= 0.0f && qx1 <= xmax && qy1 >= 0.0f && qy1 <= ymax;
+  const float flx0 = floorf(qx0), fly0 = floorf(qy0), flx1 = floorf(qx1), fly1 = floorf(qy1);
+  // taps of weight exactly 0, decided per warp so that each branch stays straight-line code: a
+  // warp whose valid pixels all have an integral motion component in y (and x), as under a
+  // static camera or an axis-aligned pan, reads 2 (1) taps instead of 4
+  const bool fy_0 = __all_sync(0xffffffffu, (!in.valid0 || qy0 == fly0) && (!in.valid1 || qy1 == fly1));
+  const bool fx_0 = __all_sync(0xffffffffu, (!in.valid0 || qx0 == flx0) && (!in.valid1 || qx1 == flx1));
+  const bool any = __any_sync(0xffffffffu, in.valid0 || in.valid1);
+  const int x0a = (int)flx0, y0a = (int)fly0, x0b = (int)flx1, y0b = (int)fly1;
+  int lo_x = 0x7fffffff, hi_x = -1, lo_y = 0x7fffffff, hi_y = -1;
+  if (in.valid0) { lo_x = x0a; hi_x = x0a; lo_y = y0a; hi_y = y0a; }
+  if (in.valid1) { lo_x = min(lo_x, x0b); hi_x = max(hi_x, x0b); lo_y = min(lo_y, y0b); hi_y = max(hi_y, y0b); }
+  lo_x = __reduce_min_sync(0xffffffffu, lo_x);
+  hi_x = __reduce_max_sync(0xffffffffu, hi_x);
+  lo_y = __reduce_min_sync(0xffffffffu, lo_y);
+  hi_y = __reduce_max_sync(0xffffffffu, hi_y);
+  if constexpr (PERSIST) __syncthreads();  // the previous tile is done with shared memory
+  if (tx == 0) sm.red[ty] = make_int4(lo_x, hi_x, lo_y, hi_y);
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kPairThreads / 32; ++w) {
+    const int4 r = sm.red[w];
+    lo_x = min(lo_x, r.x); hi_x = max(hi_x, r.y);
+    lo_y = min(lo_y, r.z); hi_y = max(hi_y, r.w);
+  }
+  const int X0 = lo_x & ~(SV::kAlignX - 1), Y0 = lo_y;  // TMA box origin: 16-byte aligned column
+  const bool fits = stage_ok && hi_x >= 0 && min(hi_x + 1, W - 1) - X0 < kStageW && min(hi_y + 1, H - 1) - Y0 < kStageH;
+  if (fits && threadIdx.x == 0) {
+    fence_proxy_async();
+    mbar_expect_tx(bar, SV::kTxBytes);
+    if (!kp.debug_withhold_copy) tma_load_3d(sm.stage, &maps->planes, X0, Y0, 0, bar);
+  }
+  // radiance tile with a 1-pixel halo: a warp takes whole rows, the left-over columns last
+  constexpr int NW = kPairThreads / 32, RH = kTH + 2, RX = kTW / 32;
+#pragma unroll
+  for (int r = 0; r < (RH + NW - 1) / NW; ++r) {
+    const int ly = ty + r * NW;
+    if (ly < RH) {
+#pragma unroll
+      for (int c = 0; c < RX; ++c) {
+        const Rgb v = load_radiance(rad, npix, bx0 - 1 + tx + 32 * c, by0 - 1 + ly, W, H);
+        sm.rad[0][ly][tx + 32 * c] = v.r;
+        sm.rad[1][ly][tx + 32 * c] = v.g;
+        sm.rad[2][ly][tx + 32 * c] = v.b;
+      }
+    }
+  }
+  if (ty == NW - 1 && tx < 2 * RH) {
+    const int ly = tx >> 1, lx = kTW + (tx & 1);
+    const Rgb v = load_radiance(rad, npix, bx0 - 1 + lx, by0 - 1 + ly, W, H);
+    sm.rad[0][ly][lx] = v.r;
+    sm.rad[1][ly][lx] = v.g;
+    sm.rad[2][ly][lx] = v.b;
+  }
+  __syncthreads();
+  const int lx0 = tx, ly0 = ty, lx1 = tx, ly1 = ty + kPairY;  // window position - 1
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float l0 = INFINITY, h0 = -INFINITY, l1 = INFINITY, h1 = -INFINITY;
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+      for (int dx = 0; dx < 3; ++dx) {
+        const float a = sm.rad[c][ly0 + dy][lx0 + dx], b = sm.rad[c][ly1 + dy][lx1 + dx];
+        l0 = fminf(l0, a);
+        h0 = fmaxf(h0, a);
+        l1 = fminf(l1, b);
+        h1 = fmaxf(h1, b);
+        if (dy == 1 && dx == 1) in.I[c] = make_float2(a, b);
+      }
+    in.lo[c] = make_float2(l0, l1);
+    in.hi[c] = make_float2(h0, h1);
+  }
+  in.miss0 = in.I[0].x != in.I[0].x;
+  in.miss1 = in.I[0].y != in.I[0].y;
+  in.missing = __any_sync(0xffffffffu, in.miss0 || in.miss1);
+  in.restart = !__all_sync(0xffffffffu, in.valid0 && in.valid1);
+  if (in.missing) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if (in.miss0) in.I[c].x = 0.0f;
+      if (in.miss1) in.I[c].y = 0.0f;
+      // no sample in the neighbourhood: no clamp
+      if (!(in.lo[c].x <= in.hi[c].x)) { in.lo[c].x = -INFINITY; in.hi[c].x = INFINITY; }
+      if (!(in.lo[c].y <= in.hi[c].y)) { in.lo[c].y = -INFINITY; in.hi[c].y = INFINITY; }
+    }
+  }
+  PairTaps t;
+  {
+    const float fx0 = qx0 - flx0, fy0 = qy0 - fly0, fx1 = qx1 - flx1, fy1 = qy1 - fly1;
+    const float2 gx = make_float2(1.0f - fx0, 1.0f - fx1), gy = make_float2(1.0f - fy0, 1.0f - fy1);
+    const float2 fx = make_float2(fx0, fx1), fy = make_float2(fy0, fy1);
+    t.w[0] = f2mul(gx, gy);
+    t.w[1] = f2mul(fx, gy);
+    t.w[2] = f2mul(gx, fy);
+    t.w[3] = f2mul(fx, fy);
+    // offsets in the window or in a plane of the copy; a restarted pixel reads offset 0
+    const int px = fits ? X0 : 0, py = fits ? Y0 : 0, row = fits ? kStageW : prev.pitch;
+    auto offs = [&](bool v, int x0, int y0, int o[4]) {
+      const int b = v ? (y0 - py) * row + x0 - px : 0;
+      const int dx = v && x0 < W - 1 ? 1 : 0, dy = v && y0 < H - 1 ? row : 0;
+      o[0] = b;
+      o[1] = b + dx;
+      o[2] = b + dy;
+      o[3] = b + dy + dx;
+    };
+    offs(in.valid0, x0a, y0a, t.o0);
+    offs(in.valid1, x0b, y0b, t.o1);
+  }
+  const uint32_t i = (uint32_t)ya * next.pitch + xa, i1 = (uint32_t)kPairY * next.pitch;
+  if (fits) {
+    bool ok = mbar_wait_bounded(bar, phase);
+    if constexpr (PERSIST) ok = !__syncthreads_or(!ok);
+    if (!ok) {
+      atomicExch(err, (int)WRLS_ERR_TIMEOUT);
+      mbar_wait_bounded(bar, phase);  // the copy may still be in flight
+      return false;
+    }
+    phase ^= 1u;
+    if (any) {
+      const StagedTaps src{reinterpret_cast<const uint32_t*>(sm.stage)};
+      if (fy_0 && fx_0) update_pair<SV, 1>(kp, src, t, in, next, i, i1, in0, in1);
+      else if (fy_0) update_pair<SV, 2>(kp, src, t, in, next, i, i1, in0, in1);
+      else update_pair<SV, 4>(kp, src, t, in, next, i, i1, in0, in1);
+      return true;
+    }
+  }
+  const GlobalTaps src{reinterpret_cast<const uint32_t*>(prev.base), prev.plane_stride};
+  if (any) update_pair<SV, 4>(kp, src, t, in, next, i, i1, in0, in1);
+  else if (in0 || in1) update_pair<SV, 0>(kp, src, t, in, next, i, i1, in0, in1);
+  return true;
+}
+
+// One tile of either form; a kernel of update_threads<SV>() threads calls it.
+template <class SV>
+constexpr int update_threads() { return SV::kScaled ? kPairThreads : kTileThreads; }
+// CTAs per SM the update is compiled for, measured at 1080p (us a frame, per-frame entry and
+// sequence entry): BF16 pairs 5 (96 registers) 72.0 / 118.8, 6 (80 registers, a small spill) 68.5 /
+// 113.6, 7 (72) 67.8 / 114.7, 8 (64, spills) slower; binary32 with 44 KB of shared memory a CTA 5 (48
+// registers) 83.1 against 88.0 at 4.
+template <class SV>
+constexpr int update_min_ctas() { return SV::kScaled ? 6 : 5; }
+template <class SV, bool PERSIST, class... A>
+__device__ __forceinline__ bool update_any(A&&... a) {
+  if constexpr (SV::kScaled) return update_tile<SV, PERSIST>(a...);
+  else return update_tile(a...);
 }
 
 // 128-byte aligned view of a dynamic shared-memory buffer.
