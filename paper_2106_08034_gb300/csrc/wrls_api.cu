@@ -100,6 +100,38 @@ bool encode_stage_maps(StateDesc& d, const char** why) {
   return true;
 }
 
+bool encode_ext_maps(StateDesc& s, int d, const char** why) {
+  s.stage_ok = false;
+  s.ext_tma_ok = false;
+  memset(&s.esmaps, 0, sizeof(s.esmaps));
+  memset(&s.emaps, 0, sizeof(s.emaps));
+  if (s.pitch < kStageW || s.H < kStageH) return true;  // smaller images use plain loads
+  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc) { *why = "cuTensorMapEncodeTiled is not available from the driver"; return false; }
+  const cuuint64_t dims[3] = {(cuuint64_t)s.pitch, (cuuint64_t)s.H, (cuuint64_t)s.nplanes};
+  const cuuint64_t strides[2] = {(cuuint64_t)s.pitch * 4, (cuuint64_t)s.plane_stride * 4};
+  const cuuint32_t es[3] = {1, 1, 1};
+  auto encode = [&](CUtensorMap* m, int w, int h, int planes) {
+    const cuuint32_t bx[3] = {(cuuint32_t)w, (cuuint32_t)h, (cuuint32_t)planes};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, s.base, dims, strides, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  if (encode(&s.esmaps.beta, kStageW, kStageH, 3 * d) != CUDA_SUCCESS ||
+      encode(&s.esmaps.p, kStageW, kStageH, d * (d + 1) / 2) != CUDA_SUCCESS ||
+      encode(&s.esmaps.z, kStageW, kStageH, 3) != CUDA_SUCCESS) {
+    *why = "cuTensorMapEncodeTiled failed for the extended state planes";
+    return false;
+  }
+  s.stage_ok = true;
+  if (s.pitch < kBlendBoxW2 || s.H < 12) return true;
+  if (encode(&s.emaps.beta, kBlendBoxW2, 12, 3 * d) != CUDA_SUCCESS || encode(&s.emaps.z, kBlendBoxW2, 12, 3) != CUDA_SUCCESS) {
+    *why = "cuTensorMapEncodeTiled failed for the extended blend window";
+    return false;
+  }
+  s.ext_tma_ok = true;
+  return true;
+}
+
 bool make_kparams(const wrls_params& p, KParams* kp, const char** why) {
   if (p.struct_size != sizeof(wrls_params)) { *why = "params.struct_size != sizeof(wrls_params)"; return false; }
   if (!(p.lambda > 0.0f && p.lambda <= 1.0f)) { *why = "lambda must be in (0, 1]"; return false; }
@@ -246,7 +278,7 @@ static wrls_status enqueue_update(wrls_stream* s, const float* radiance, const f
   if (s->ext)
     e = launch_ext_update(s->ep, s->dim, prev, next, s->need_reset, radiance, motion,
                           s->prm.weight_mode == 2 ? variance : nullptr, s->prm.n_gbuf > 0 ? features : nullptr,
-                          s->cs);
+                          s->err, s->cs);
   else
     e = launch_update(s->kp, prev, next, s->need_reset, radiance, motion, s->err, s->cs);
   if (e != cudaSuccess) {
@@ -264,7 +296,7 @@ static wrls_status enqueue_blend(wrls_stream* s, const KParams& kp, const float*
   if (s->ext) {
     ExtParams ep = s->ep;
     ep.kp = kp;
-    e = launch_ext_blend(ep, s->dim, next, s->prm.n_gbuf > 0 ? features : nullptr, out, cs);
+    e = launch_ext_blend(ep, s->dim, next, s->prm.n_gbuf > 0 ? features : nullptr, out, s->err, cs);
   } else {
     e = launch_blend(kp, s->blend_cfg, next, out, s->err, cs);
   }
@@ -290,7 +322,7 @@ static bool add_third_copy(wrls_stream* s) {
   StateDesc d = s->state[0];
   d.base = mem;
   const char* why = "";
-  if (!s->ext && !encode_stage_maps(d, &why)) {
+  if (!(s->ext ? encode_ext_maps(d, s->dim, &why) : encode_stage_maps(d, &why))) {
     cudaFree(mem);
     return false;
   }
@@ -400,7 +432,7 @@ wrls_status wrls_stream_create(int width, int height, const wrls_params* p, wrls
     d.pitch = pitch;
     d.plane_stride = ps;
     d.nplanes = nplanes;
-    if (!ext && !encode_stage_maps(d, &why)) {
+    if (!(ext ? encode_ext_maps(d, dim, &why) : encode_stage_maps(d, &why))) {
       cudaFree(s->mem);
       set_error("wrls_stream_create: %s", why);
       delete s;

@@ -140,6 +140,17 @@ struct BlendMaps {
   CUtensorMap beta16w, z16w, beta8w, z8w;  // 72-column boxes
 };
 
+// Tensor maps of the extended path's blend window: boxes of kBlendBoxW2 columns x 12 rows of the
+// 3d beta planes and the 3 z planes.
+struct ExtMaps {
+  CUtensorMap beta, z;
+};
+// Tensor maps of the extended path's staged update window: boxes of kStageW x kStageH of the three
+// sections of the state.
+struct ExtStageMaps {
+  CUtensorMap beta, p, z;
+};
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }

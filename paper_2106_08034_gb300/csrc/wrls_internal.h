@@ -23,6 +23,9 @@ struct StateDesc {
   StageMaps maps{};          // TMA tensor map of this copy's planes
   bool stage_ok = false;     // maps encoded and the image is at least one staging box
   BlendMaps bmaps{};         // TMA tensor maps of the blend windows
+  ExtStageMaps esmaps{};     // extended path: TMA tensor maps of the update's window
+  ExtMaps emaps{};           // extended path: TMA tensor maps of the blend window
+  bool ext_tma_ok = false;   // extended path: maps encoded (image >= one 72 x 12 box)
   bool blend_tma_ok = false; // 40-column blend maps encoded (binary32 state, image >= one box)
   bool blend_tma2_ok = false; // 72-column blend maps encoded
 
@@ -51,10 +54,13 @@ inline bool uses_ext(const wrls_params& p) { return p.n_gbuf > 0 || p.weight_mod
 int ext_dim(const wrls_params& p);  // predictor dimension d
 int ext_planes(int d);              // state planes of dimension d: 3d + d(d+1)/2 + 3
 cudaError_t launch_ext_update(const ExtParams& ep, int d, const StateDesc& prev, const StateDesc& next, bool reset,
-                              const float* rad, const float* mot, const float* var, const float* gbuf,
+                              const float* rad, const float* mot, const float* var, const float* gbuf, int* err,
                               cudaStream_t cs);
-cudaError_t launch_ext_blend(const ExtParams& ep, int d, const StateDesc& cur, const float* gbuf, float* out,
+cudaError_t launch_ext_blend(const ExtParams& ep, int d, const StateDesc& cur, const float* gbuf, float* out, int* err,
                              cudaStream_t cs);
+// Encode the tensor maps of an extended state copy of predictor dimension d (sets stage_ok and
+// ext_tma_ok; false only on a driver error).
+bool encode_ext_maps(StateDesc& s, int d, const char** why);
 cudaError_t launch_read_state_ext(const StateDesc& cur, int nplanes, float* dst, cudaStream_t cs);
 cudaError_t launch_write_state_ext(const StateDesc& cur, int nplanes, const float* src, cudaStream_t cs);
 

@@ -156,3 +156,24 @@ def test_extended_streams_are_rejected_by_batched_ticks():
         s.denoise(x, m, o)
     W.wrls_batch_destroy(b)
     s.close()
+
+
+# the staged window is 40 x 10, the blend window 72 x 12 (tiles of 64 x 8): exactly one of them, one
+# less, tiles cut on each side, images without a window
+@pytest.mark.parametrize("wh", [(72, 12), (73, 13), (65, 11), (64, 12), (40, 10), (33, 9), (129, 21), (1, 1)])
+@pytest.mark.parametrize("kw", [dict(n_gbuf=4), dict(n_gbuf=1), dict(weight_mode=2, feature_mode=1),
+                                dict(reproj_filter=1, n_gbuf=2)])
+@pytest.mark.parametrize("motion", ["orbit", "scatter"])
+def test_tile_edges(wh, kw, motion):
+    """Sizes at the edges of the staged and blend windows; "scatter" moves every pixel by up to
+    20 pixels on its own, so that the taps are read from global memory."""
+    w, h = wh
+    spec = synth.SceneSpec(w, h, 4, seed=52, motion="orbit", firefly_frac=0.05)
+
+    def hooks(t, rad, mot, var, feat):
+        if motion == "scatter":
+            g = torch.Generator().manual_seed(53 + t)
+            mot = 40 * (torch.rand(2, h, w, generator=g) - 0.5)
+            rad[0, :2, :3] = float("nan")
+        return rad, mot, var, feat
+    run_ext(cpu_frames(spec), w, h, params(**kw), hooks=hooks)
