@@ -179,7 +179,7 @@ bool make_kparams(const wrls_params& p, KParams* kp, const char** why) {
   kp->feature_mode = p.feature_mode;
   kp->init_mode = p.init_mode;
   kp->debug_withhold_copy = 0;
-  kp->blend_ctas_cap = 0;
+  kp->hints = 0;
   return true;
 }
 
@@ -270,17 +270,19 @@ static wrls_status timing_slot(wrls_stream* s, cudaEvent_t** ev) {
 }
 
 // Update of the next frame (state copy cur -> next_copy) on the stream's CUDA stream.
-static wrls_status enqueue_update(wrls_stream* s, const float* radiance, const float* variance,
+static wrls_status enqueue_update(wrls_stream* s, const KParams& kp, const float* radiance, const float* variance,
                                   const float* features, const float* motion, const char* who) {
   const StateDesc& prev = s->state[s->cur];
   const StateDesc& next = s->state[next_copy(s)];
   cudaError_t e;
-  if (s->ext)
-    e = launch_ext_update(s->ep, s->dim, prev, next, s->need_reset, radiance, motion,
+  if (s->ext) {
+    ExtParams ep = s->ep;
+    ep.kp = kp;
+    e = launch_ext_update(ep, s->dim, prev, next, s->need_reset, radiance, motion,
                           s->prm.weight_mode == 2 ? variance : nullptr, s->prm.n_gbuf > 0 ? features : nullptr,
                           s->err, s->cs);
-  else
-    e = launch_update(s->kp, prev, next, s->need_reset, radiance, motion, s->err, s->cs);
+  } else
+    e = launch_update(kp, prev, next, s->need_reset, radiance, motion, s->err, s->cs);
   if (e != cudaSuccess) {
     set_error("%s: update kernel launch: %s", who, cudaGetErrorString(e));
     return WRLS_ERR_CUDA;
@@ -439,12 +441,14 @@ wrls_status wrls_stream_create(int width, int height, const wrls_params* p, wrls
       return WRLS_ERR_CUDA;
     }
   }
-  // Default blend configuration, from the measured ranking: on images of at least 2^19 pixels
-  // the two-wide packed blend, 64 x 8 tiles (9) for the binary32 state, 64 x 16 tiles (8) for
-  // the 16-bit formats (some 1000 tiles, several per SM); on smaller images the
-  // one-CTA-per-tile 16 x 2 blend (2), where one tile per CTA spreads the work over more SMs.
+  // Default blend configuration, from the measured ranking (us a frame through per-frame calls with
+  // the one-CTA-per-tile 16 x 2 blend (2) / the two-wide one): on images of at least 2^17 pixels the
+  // two-wide packed blend, 64 x 8 tiles (9) for the binary32 state (512x512 25.7 / 23.0, 643x361 24.3 /
+  // 22.1, 1080p 159.5 / 138.8), 64 x 16 tiles (8) for the 16-bit formats (512x512 20.8 / 19.6, 643x361 20.1 /
+  // 19.4, 1080p 133.2 / 130.0); on smaller images 2, where one tile per CTA spreads the work over more
+  // SMs (128x128 8.3 / 8.9, BF16 7.8 / 10.1; at 256x256 the two are within 5 %).
   if (!ext) {
-    const bool big = (long long)width * height >= (1ll << 19);
+    const bool big = (long long)width * height >= (1ll << 17);
     s->blend_cfg = (big && s->state[0].blend_tma2_ok) ? (p->state_precision == 0 ? 9 : 8) : 2;
   }
   *out = s;
@@ -467,13 +471,18 @@ wrls_status wrls_denoise_frame(wrls_stream* s, const float* radiance, const floa
   st = timing_slot(s, &ev);
   if (st != WRLS_OK) return st;
   if (ev) WRLS_CHECK_CUDA(cudaEventRecord(ev[0], s->cs), "wrls_denoise_frame: event record");
-  st = enqueue_update(s, radiance, variance, features, motion, "wrls_denoise_frame");
+  KParams kp = s->kp;
+  // each kernel is set up while the one before finishes (not under stream capture)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s->cs, &cap) != cudaSuccess) cudaGetLastError();
+  else if (cap == cudaStreamCaptureStatusNone) kp.hints |= kHintPdl;
+  st = enqueue_update(s, kp, radiance, variance, features, motion, "wrls_denoise_frame");
   if (st != WRLS_OK) return st;
   if (ev) {
     WRLS_CHECK_CUDA(cudaEventRecord(ev[1], s->cs), "wrls_denoise_frame: event record");
     WRLS_CHECK_CUDA(cudaEventRecord(ev[2], s->cs), "wrls_denoise_frame: event record");
   }
-  st = enqueue_blend(s, s->kp, features, out, s->cs, "wrls_denoise_frame");
+  st = enqueue_blend(s, kp, features, out, s->cs, "wrls_denoise_frame");
   if (st != WRLS_OK) return st;
   if (ev) {
     WRLS_CHECK_CUDA(cudaEventRecord(ev[3], s->cs), "wrls_denoise_frame: event record");
@@ -528,7 +537,7 @@ wrls_status wrls_denoise_sequence(wrls_stream* s, const wrls_frame_io* frames, i
     if (st0 != WRLS_OK) return st0;
   }
   KParams kpo = s->kp;
-  kpo.blend_ctas_cap = s->overlap_ctas;
+  kpo.hints = s->overlap_ctas;
   wrls_status st = WRLS_OK;
   auto ck = [&](cudaError_t e, const char* what) {
     if (e != cudaSuccess && st == WRLS_OK) {
@@ -546,7 +555,7 @@ wrls_status wrls_denoise_sequence(wrls_stream* s, const wrls_frame_io* frames, i
     cudaEvent_t* ev = nullptr;
     if ((st = timing_slot(s, &ev)) != WRLS_OK) break;
     if (ev && !ck(cudaEventRecord(ev[0], s->cs), "event record")) break;
-    if ((st = enqueue_update(s, f.radiance, f.variance, f.features, f.motion, "wrls_denoise_sequence")) != WRLS_OK)
+    if ((st = enqueue_update(s, kpo, f.radiance, f.variance, f.features, f.motion, "wrls_denoise_sequence")) != WRLS_OK)
       break;
     if (ev && !ck(cudaEventRecord(ev[1], s->cs), "event record")) break;
     if (!ck(cudaEventRecord(s->ev_u, s->cs), "event record")) break;
@@ -625,7 +634,7 @@ wrls_status wrls_denoise_sequence_host(wrls_stream* s, const wrls_frame_io* fram
     WRLS_CHECK_CUDA(cudaStreamSynchronize(s->cs), "wrls_denoise_sequence_host: synchronize");
   }
   KParams kpo = s->kp;
-  kpo.blend_ctas_cap = s->overlap_ctas;
+  kpo.hints = s->overlap_ctas;
   auto ck = [&](cudaError_t e, const char* what) {
     if (e != cudaSuccess && st == WRLS_OK) {
       set_error("wrls_denoise_sequence_host: %s: %s", what, cudaGetErrorString(e));
@@ -660,7 +669,7 @@ wrls_status wrls_denoise_sequence_host(wrls_stream* s, const wrls_frame_io* fram
     const int nc = s->ncopies;
     if (i >= nc && !ck(cudaStreamWaitEvent(s->cs, s->ev_b[(i - nc) % 3], 0), "wait")) break;
     if (!ck(cudaStreamWaitEvent(s->cs, s->ev_in[k], 0), "wait")) break;
-    if ((st = enqueue_update(s, d_rad, d_var, d_g, d_mot, "wrls_denoise_sequence_host")) != WRLS_OK) break;
+    if ((st = enqueue_update(s, kpo, d_rad, d_var, d_g, d_mot, "wrls_denoise_sequence_host")) != WRLS_OK) break;
     if (!ck(cudaEventRecord(s->ev_u, s->cs), "event record")) break;
     // blend on the side stream (after the update, and after the output copy of frame i - NS)
     if (!ck(cudaStreamWaitEvent(s->side, s->ev_u, 0), "wait")) break;

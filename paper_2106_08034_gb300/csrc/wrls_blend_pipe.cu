@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kTW * TH / R)
     mbar_init(&bar[1], 1);
   }
   __syncthreads();
+  pdl_wait();
   uint32_t ph0 = 0u, ph1 = 0u;  // phases of the two windows' mbarriers
   if (threadIdx.x == 0) {
     mbar_expect_tx(&bar[0], G::kTx);
@@ -136,6 +137,7 @@ __global__ void __launch_bounds__(kTW * TH / R)
     const int b = NBUF == 2 ? (it & 1) : 0;
     float* wcur = sm + b * G::BUF;
     const int next = tile + gridDim.x;
+    if (next >= n_tiles) pdl_next();
     if (NBUF == 2 && next < n_tiles && threadIdx.x == 0) {  // the other window was released by the last barrier
       float* wn = sm + (b ^ 1) * G::BUF;
       fence_proxy_async();
@@ -197,11 +199,10 @@ static cudaError_t launch_tma_cfg(const KParams& kp, const StateDesc& cur, float
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int n_tiles = ((cur.W + kTW - 1) / kTW) * ((cur.H + TH - 1) / TH);
-  const int use = (kp.blend_ctas_cap > 0 && kp.blend_ctas_cap < per_sm) ? kp.blend_ctas_cap : per_sm;
+  const int use = (hint_ctas(kp) > 0 && hint_ctas(kp) < per_sm) ? hint_ctas(kp) : per_sm;
   int grid = sms * use;
   if (grid > n_tiles) grid = n_tiles;
-  k_blend_tma<TH, R, MODE, NBUF><<<grid, nt, bytes, cs>>>(kp, cur.W, cur.H, cur.bmaps, out, err);
-  return cudaGetLastError();
+  return launch_kernel(k_blend_tma<TH, R, MODE, NBUF>, grid, nt, bytes, cs, hint_pdl(kp), kp, cur.W, cur.H, cur.bmaps, out, err);
 }
 
 template <int MODE>
@@ -473,6 +474,7 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
   if (tile >= n_tiles) return;
   if (threadIdx.x == 0) mbar_init(&bar, 1);
   __syncthreads();
+  pdl_wait();
   uint32_t ph = 0u;
   if (threadIdx.x == 0) {
     mbar_expect_tx(&bar, G::kTx);
@@ -481,6 +483,7 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
   }
   for (;;) {
     const int next = tile + gridDim.x;
+    if (next >= n_tiles) pdl_next();
     const bool ok = mbar_wait_bounded(&bar, ph);
     if (__syncthreads_or(!ok)) {
       if (threadIdx.x == 0) atomicExch(err, (int)WRLS_ERR_TIMEOUT);
@@ -544,11 +547,10 @@ static cudaError_t launch_tma2_cfg(const KParams& kp, const StateDesc& cur, floa
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int n_tiles = ((cur.W + 2 * kTW - 1) / (2 * kTW)) * ((cur.H + TH - 1) / TH);
-  const int use = (kp.blend_ctas_cap > 0 && kp.blend_ctas_cap < per_sm) ? kp.blend_ctas_cap : per_sm;
+  const int use = (hint_ctas(kp) > 0 && hint_ctas(kp) < per_sm) ? hint_ctas(kp) : per_sm;
   int grid = sms * use;
   if (grid > n_tiles) grid = n_tiles;
-  k_blend_tma2<TH, R, MODE><<<grid, nt, bytes, cs>>>(kp, cur.W, cur.H, cur.bmaps, out, err);
-  return cudaGetLastError();
+  return launch_kernel(k_blend_tma2<TH, R, MODE>, grid, nt, bytes, cs, hint_pdl(kp), kp, cur.W, cur.H, cur.bmaps, out, err);
 }
 
 // ---- two-wide variant for the 16-bit state formats ---------------------------------------
@@ -599,6 +601,7 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
   if (tile >= n_tiles) return;
   if (threadIdx.x == 0) mbar_init(&bar, 1);
   __syncthreads();
+  pdl_wait();
   uint32_t ph = 0u;
   if (threadIdx.x == 0) {
     mbar_expect_tx(&bar, G::kTx);
@@ -607,6 +610,7 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
   }
   for (;;) {
     const int next = tile + gridDim.x;
+    if (next >= n_tiles) pdl_next();
     const bool ok = mbar_wait_bounded(&bar, ph);
     if (__syncthreads_or(!ok)) {
       if (threadIdx.x == 0) atomicExch(err, (int)WRLS_ERR_TIMEOUT);
@@ -709,11 +713,10 @@ static cudaError_t launch_tma2h_cfg(const KParams& kp, const StateDesc& cur, flo
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int n_tiles = ((cur.W + 2 * kTW - 1) / (2 * kTW)) * ((cur.H + TH - 1) / TH);
-  const int use = (kp.blend_ctas_cap > 0 && kp.blend_ctas_cap < per_sm) ? kp.blend_ctas_cap : per_sm;
+  const int use = (hint_ctas(kp) > 0 && hint_ctas(kp) < per_sm) ? hint_ctas(kp) : per_sm;
   int grid = sms * use;
   if (grid > n_tiles) grid = n_tiles;
-  k_blend_tma2h<TH, R, MODE, T><<<grid, nt, bytes, cs>>>(kp, cur.W, cur.H, cur.bmaps, out, err);
-  return cudaGetLastError();
+  return launch_kernel(k_blend_tma2h<TH, R, MODE, T>, grid, nt, bytes, cs, hint_pdl(kp), kp, cur.W, cur.H, cur.bmaps, out, err);
 }
 
 template <typename T>

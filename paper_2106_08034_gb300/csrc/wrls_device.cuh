@@ -42,8 +42,14 @@ struct KParams {
   int feature_mode;
   int init_mode;
   int debug_withhold_copy;  // test hook: arm the state-window barrier without issuing the copy
-  int blend_ctas_cap;       // host-side launch hint: CTAs per SM of the persistent blends (0 = all that fit)
+  // host-side launch hints: bits 0-7 CTAs per SM of the persistent blends (0 = all that fit), bit 8
+  // start beside the tail of the kernel before (pdl_wait)
+  int hints;
 };
+
+constexpr int kHintPdl = 1 << 8;
+__host__ __device__ inline int hint_ctas(const KParams& kp) { return kp.hints & 0xff; }
+__host__ __device__ inline bool hint_pdl(const KParams& kp) { return (kp.hints & kHintPdl) != 0; }
 
 // 2^x on the SFU (PTX ex2.approx, max relative error about 2^-22).
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -66,6 +72,19 @@ __device__ __forceinline__ float blend_rk(float z0, float z1, float z2, float ep
   const float r = 1.0f / (sqrtf(fmaf(z2, z2, fmaf(z1, z1, z0 * z0))) + eps);
   return r * r * range_k;
 }
+
+// Programmatic dependent launch: a frame's kernels run one after the other, and the next one may be
+// set up on the SMs while the last CTAs of the one before finish. pdl_next() lets it (once every
+// CTA of this kernel has called it or ended); pdl_wait() then holds it until the kernel before has completed
+// and its writes are visible, so nothing of global memory is touched ahead of it. Both do nothing
+// in a kernel launched without the attribute. pdl_next() stands where a CTA has its data and is
+// about to compute (persistent blends: before their last tile): called at the start of the
+// kernels, waiting CTAs of the kernels after took slots early and were placed unevenly (256x256
+// 16.4 -> 20.8 us a frame, 1080p 144 -> 149). Per-frame calls, us a frame: 128x128 12.3 -> 7.7, 643x361
+// 28.7 -> 22.1 (with the two-wide blend), 1280x720 72.1 -> 67.3, 1080p 142.4 -> 135.9, FP16 1440p 214.6 ->
+// 208.6.
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- packed binary32 pairs (sm_100 family: one instruction for two lanes' worth) ----------
 // Each component is rounded as the scalar operation would be (round to nearest even, no

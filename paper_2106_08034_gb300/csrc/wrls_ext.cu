@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
   __shared__ int4 red[kExtTH];
   __shared__ alignas(8) uint64_t bar[3];
   if (threadIdx.x < 3) mbar_init(&bar[threadIdx.x], 1);
+  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int x = blockIdx.x * kExtTW + lane, y = blockIdx.y * kExtTH + warp;
   const bool inside = x < W && y < H;
@@ -287,6 +288,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
     lo_x = min(lo_x, r.x); hi_x = max(hi_x, r.y);
     lo_y = min(lo_y, r.z); hi_y = max(hi_y, r.w);
   }
+  pdl_next();
   const int more = nearest ? 0 : 1;
   const int X0 = lo_x & ~3, Y0 = lo_y;  // TMA box origin: 16-byte aligned column
   const bool fits = stage_ok && hi_x >= 0 && min(hi_x + more, W - 1) - X0 < kStageW && min(hi_y + more, H - 1) - Y0 < kStageH;
@@ -406,6 +408,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH / kExtBlendRows)
   const KParams& kp = ep.kp;
   const int bx0 = blockIdx.x * kExtTW, by0 = blockIdx.y * kExtTH;
   const int tid = threadIdx.y * kExtTW + threadIdx.x;
+  pdl_wait();
   for (int e = tid; e < kExtSP; e += NT) {
     const int gx = bx0 - 2 + e % kExtSW, gy = by0 - 2 + e / kExtSW;
     if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
@@ -429,6 +432,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH / kExtBlendRows)
     }
   }
   __syncthreads();
+  pdl_next();
   const int x = bx0 + threadIdx.x;
   const int ty0 = threadIdx.y * kExtBlendRows;  // first of the thread's two rows in the tile
   const size_t npix = (size_t)W * H;
@@ -546,6 +550,7 @@ __global__ void __launch_bounds__(128)
   const KParams& kp = ep.kp;
   const int bx0 = blockIdx.x * kExt2W, by0 = blockIdx.y * kExt2H;
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  pdl_wait();
   if (threadIdx.x == 0) {
     mbar_init(&zbar, 1);
     mbar_init(&bbar, 1);
@@ -593,6 +598,7 @@ __global__ void __launch_bounds__(128)
     mbar_wait_bounded(&bbar, 0);
     return;
   }
+  pdl_next();
   float2 zi[2][3], ri[2], den[2], acc[2][3];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
@@ -702,10 +708,9 @@ static cudaError_t launch_ext_t(const ExtParams& ep, const StateDesc& prev, cons
     attr_set = true;
   }
   const dim3 grid((prev.W + kExtTW - 1) / kExtTW, (prev.H + kExtTH - 1) / kExtTH);
-  k_update_ext<D, F><<<grid, kExtTW * kExtTH, bytes, cs>>>(ep, prev.W, prev.H, reset ? 1 : 0, prev.stage_ok ? 1 : 0,
-                                                           (const float*)prev.base, (float*)next.base, prev.pitch,
-                                                           prev.plane_stride, prev.esmaps, rad, mot, var, gbuf, err);
-  return cudaGetLastError();
+  return launch_kernel(k_update_ext<D, F>, grid, kExtTW * kExtTH, bytes, cs, hint_pdl(ep.kp), ep, prev.W, prev.H, reset ? 1 : 0,
+                       prev.stage_ok ? 1 : 0, (const float*)prev.base, (float*)next.base, prev.pitch, prev.plane_stride,
+                       prev.esmaps, rad, mot, var, gbuf, err);
 }
 
 template <int D, bool F>
@@ -720,13 +725,11 @@ static cudaError_t launch_ext_blend_t(const ExtParams& ep, const StateDesc& cur,
       attr_set = true;
     }
     const dim3 grid((cur.W + kExt2W - 1) / kExt2W, (cur.H + kExt2H - 1) / kExt2H);
-    k_blend_ext2<D, F><<<grid, 128, bytes, cs>>>(ep, cur.W, cur.H, cur.emaps, gbuf, out, err);
-    return cudaGetLastError();
+    return launch_kernel(k_blend_ext2<D, F>, grid, 128, bytes, cs, hint_pdl(ep.kp), ep, cur.W, cur.H, cur.emaps, gbuf, out, err);
   }
   const dim3 grid((cur.W + kExtTW - 1) / kExtTW, (cur.H + kExtTH - 1) / kExtTH);
-  k_blend_ext<D, F><<<grid, dim3(kExtTW, kExtTH / kExtBlendRows), 0, cs>>>(ep, cur.W, cur.H, (const float*)cur.base, cur.pitch,
-                                            cur.plane_stride, gbuf, out);
-  return cudaGetLastError();
+  return launch_kernel(k_blend_ext<D, F>, grid, dim3(kExtTW, kExtTH / kExtBlendRows), 0, cs, hint_pdl(ep.kp), ep, cur.W, cur.H,
+                       (const float*)cur.base, cur.pitch, cur.plane_stride, gbuf, out);
 }
 
 int ext_dim(const wrls_params& p) { return (p.feature_mode == 0 ? 4 : 1) + p.n_gbuf; }

@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(update_threads<SV>(), update_min_ctas<SV>())
   __shared__ alignas(8) uint64_t bar;
   UpdateSmem<SV>& sm = *reinterpret_cast<UpdateSmem<SV>*>(align128(dsmem));
   if (threadIdx.x == 0) mbar_init(&bar, 1);
+  pdl_wait();
   uint32_t phase = 0;
   update_any<SV, false>(sm, &bar, phase, err, kp, W, H, reset != 0, stage_ok != 0, prev, next, &maps, rad, mot,
                         (int)blockIdx.x * kTW, (int)blockIdx.y * kTH);
@@ -25,6 +26,7 @@ template <class SV, int TH, int R, int MODE>
 __global__ void __launch_bounds__(kTW * TH / R)
     k_blend(const KParams kp, const int W, const int H, const SV cur, float* __restrict__ out) {
   extern __shared__ float4 sm_blend[];
+  pdl_wait();
   blend_tile<SV, TH, R, MODE>(sm_blend, kp, W, H, cur, out, blockIdx.x * kTW, blockIdx.y * TH);
 }
 
@@ -63,9 +65,8 @@ static cudaError_t launch_update_t(const KParams& kp, const StateDesc& prev, con
     attr_set = true;
   }
   const dim3 grid((prev.W + kTW - 1) / kTW, (prev.H + kTH - 1) / kTH);
-  k_update<SV><<<grid, update_threads<SV>(), bytes, cs>>>(kp, prev.W, prev.H, reset ? 1 : 0, prev.stage_ok ? 1 : 0,
-                                                   pv, nx, prev.maps, rad, mot, err);
-  return cudaGetLastError();
+  return launch_kernel(k_update<SV>, grid, update_threads<SV>(), bytes, cs, hint_pdl(kp), kp, prev.W, prev.H, reset ? 1 : 0,
+                       prev.stage_ok ? 1 : 0, pv, nx, prev.maps, rad, mot, err);
 }
 
 cudaError_t launch_update(const KParams& kp, const StateDesc& prev, const StateDesc& next, bool reset,
@@ -90,8 +91,7 @@ static cudaError_t launch_blend_cfg(const KParams& kp, const SV& cur, int W, int
     attr_set = true;
   }
   const dim3 grid((W + kTW - 1) / kTW, (H + TH - 1) / TH);
-  k_blend<SV, TH, R, MODE><<<grid, kTW * TH / R, bytes, cs>>>(kp, W, H, cur, out);
-  return cudaGetLastError();
+  return launch_kernel(k_blend<SV, TH, R, MODE>, grid, kTW * TH / R, bytes, cs, hint_pdl(kp), kp, W, H, cur, out);
 }
 
 template <class SV, int MODE>

@@ -100,6 +100,22 @@ cudaError_t launch_write_state(const StateDesc& cur, const float* src, cudaStrea
 
 void set_error(const char* fmt, ...);
 
+// Launch, with the programmatic-serialisation attribute if `pdl` (kernels that call pdl_wait).
+template <class... P, class... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t cs, bool pdl, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = cs;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Return WRLS_ERR_CUDA with a message from an entry point when a CUDA call fails.
 #define WRLS_CHECK_CUDA(call, what)                      \
   do {                                                   \
