@@ -473,9 +473,7 @@ wrls_status wrls_denoise_frame(wrls_stream* s, const float* radiance, const floa
   if (ev) WRLS_CHECK_CUDA(cudaEventRecord(ev[0], s->cs), "wrls_denoise_frame: event record");
   KParams kp = s->kp;
   // each kernel is set up while the one before finishes (not under stream capture)
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s->cs, &cap) != cudaSuccess) cudaGetLastError();
-  else if (cap == cudaStreamCaptureStatusNone) kp.hints |= kHintPdl;
+  if (pdl_allowed(s->cs)) kp.hints |= kHintPdl;
   st = enqueue_update(s, kp, radiance, variance, features, motion, "wrls_denoise_frame");
   if (st != WRLS_OK) return st;
   if (ev) {

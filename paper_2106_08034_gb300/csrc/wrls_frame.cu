@@ -33,9 +33,11 @@ __global__ void __launch_bounds__(kTW * TH / R)
 template <class SV>
 __global__ void k_read_state(const int W, const int H, const SV cur, float* __restrict__ dst) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  pdl_wait();
   if (x >= W || y >= H) return;
   float v[kNState];
   cur.load((size_t)y * cur.pitch + x, v);
+  pdl_next();
   const size_t npix = (size_t)W * H, j = (size_t)y * W + x;
 #pragma unroll
   for (int p = 0; p < kNState; ++p) dst[p * npix + j] = v[p];
@@ -45,11 +47,13 @@ __global__ void k_read_state(const int W, const int H, const SV cur, float* __re
 template <class SV>
 __global__ void k_write_state(const int W, const int H, const SV cur, const float* __restrict__ src) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  pdl_wait();
   if (x >= W || y >= H) return;
   const size_t npix = (size_t)W * H, j = (size_t)y * W + x;
   float v[kNState];
 #pragma unroll
   for (int p = 0; p < kNState; ++p) v[p] = src[p * npix + j];
+  pdl_next();
   cur.store((size_t)y * cur.pitch + x, v);
 }
 
@@ -127,23 +131,21 @@ cudaError_t launch_blend(const KParams& kp, int cfg, const StateDesc& cur, float
 cudaError_t launch_write_state(const StateDesc& cur, const float* src, cudaStream_t cs) {
   const dim3 grid((cur.W + 127) / 128, cur.H);
   switch (cur.precision) {
-    case 0: k_write_state<<<grid, 128, 0, cs>>>(cur.W, cur.H, cur.f32(), src); break;
-    case 1: k_write_state<<<grid, 128, 0, cs>>>(cur.W, cur.H, cur.bf16(), src); break;
-    case 2: k_write_state<<<grid, 128, 0, cs>>>(cur.W, cur.H, cur.f16(), src); break;
-    default: return cudaErrorInvalidValue;
+    case 0: return launch_kernel(k_write_state<StateF32>, grid, 128, 0, cs, pdl_allowed(cs), cur.W, cur.H, cur.f32(), src);
+    case 1: return launch_kernel(k_write_state<StateBF16>, grid, 128, 0, cs, pdl_allowed(cs), cur.W, cur.H, cur.bf16(), src);
+    case 2: return launch_kernel(k_write_state<StateF16>, grid, 128, 0, cs, pdl_allowed(cs), cur.W, cur.H, cur.f16(), src);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_read_state(const StateDesc& cur, float* dst, cudaStream_t cs) {
   const dim3 grid((cur.W + 127) / 128, cur.H);
   switch (cur.precision) {
-    case 0: k_read_state<<<grid, 128, 0, cs>>>(cur.W, cur.H, cur.f32(), dst); break;
-    case 1: k_read_state<<<grid, 128, 0, cs>>>(cur.W, cur.H, cur.bf16(), dst); break;
-    case 2: k_read_state<<<grid, 128, 0, cs>>>(cur.W, cur.H, cur.f16(), dst); break;
-    default: return cudaErrorInvalidValue;
+    case 0: return launch_kernel(k_read_state<StateF32>, grid, 128, 0, cs, pdl_allowed(cs), cur.W, cur.H, cur.f32(), dst);
+    case 1: return launch_kernel(k_read_state<StateBF16>, grid, 128, 0, cs, pdl_allowed(cs), cur.W, cur.H, cur.bf16(), dst);
+    case 2: return launch_kernel(k_read_state<StateF16>, grid, 128, 0, cs, pdl_allowed(cs), cur.W, cur.H, cur.f16(), dst);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace wrls

@@ -100,6 +100,16 @@ cudaError_t launch_write_state(const StateDesc& cur, const float* src, cudaStrea
 
 void set_error(const char* fmt, ...);
 
+// Whether a kernel on `cs` may be launched with that attribute: not under stream capture.
+inline bool pdl_allowed(cudaStream_t cs) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(cs, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
+
 // Launch, with the programmatic-serialisation attribute if `pdl` (kernels that call pdl_wait).
 template <class... P, class... A>
 inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t cs, bool pdl, A&&... args) {

@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(128)
     k_render_vpt(const __grid_constant__ VptArgs s, const int W, const int H, const int spp, const uint32_t frame,
                  float* __restrict__ samples, float* __restrict__ world, float* __restrict__ features) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  pdl_wait();
   if (x >= W || y >= H) return;
   const size_t np = (size_t)W * H, j = (size_t)y * W + x;
   float best_t = INFINITY, by0 = 0.0f, by1 = 0.0f, by2 = 0.0f;
@@ -312,8 +313,9 @@ wrls_status wrls_render_vpt(const wrls_vpt_scene* sc, int width, int height, int
   a.albedo = sc->albedo;
   a.max_bounces = sc->max_bounces;
   const dim3 grid((width + 127) / 128, height);
-  k_render_vpt<<<grid, 128, 0, (cudaStream_t)cuda_stream>>>(a, width, height, spp, frame, samples, world, features);
-  cudaError_t e = cudaGetLastError();
+  cudaStream_t cs = (cudaStream_t)cuda_stream;
+  cudaError_t e = launch_kernel(k_render_vpt, grid, 128, 0, cs, pdl_allowed(cs), a, width, height, spp, frame, samples, world,
+                                features);
   if (e != cudaSuccess) {
     set_error("wrls_render_vpt: launch: %s", cudaGetErrorString(e));
     return WRLS_ERR_CUDA;

@@ -107,3 +107,47 @@ def test_input_steps_reject_bad_arguments():
         W.wrls_reconstruct(x, x[0, :3])              # output overlaps the samples
     with pytest.raises(W.WrlsError):
         W.wrls_velocity_from_world(r, np.full((4, 4), np.nan), torch.empty(2, 8, 8, device="cuda"))
+
+
+# tiles of 32 x 8, two rows a thread: cut after either row, one row or column, several chunks of
+# sample indices; `far` puts some offsets beyond half a pixel, so that the support is tested
+@pytest.mark.parametrize("size", [(32, 8), (33, 9), (31, 7), (64, 1), (1, 17), (95, 23)])
+@pytest.mark.parametrize("spp,radius,far", [(1, 1.5, False), (2, 1.5, True), (3, 1.2, False), (5, 0.6, True)])
+def test_reconstruction_tile_edges(size, spp, radius, far):
+    w, h = size
+    gen = torch.Generator().manual_seed(w * 100 + h + spp)
+    smp = torch.rand(spp, 5, h, w, generator=gen)
+    smp[:, 3:] -= 0.5
+    if far:
+        smp[:, 3:][torch.rand(spp, 2, h, w, generator=gen) < 0.1] *= 2.5
+    smp[:, 0][torch.rand(spp, h, w, generator=gen) < 0.1] = float("nan")
+    smp[:, 4][torch.rand(spp, h, w, generator=gen) < 0.05] = float("-inf")
+    d = smp.cuda()
+    rad, var = torch.empty(3, h, w, device="cuda"), torch.empty(h, w, device="cuda")
+    W.wrls_reconstruct(d, rad, var, W.wrls_recon_params_default(radius=radius))
+    # the support test is binary32 on both sides
+    ref, rvar = O.reconstruct(smp.numpy(), radius=float(np.float32(radius)))
+    got = rad.cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    fin = np.isfinite(ref[0])
+    # weights carry ex2's 2^-22 and the sums up to 9 spp roundings
+    assert np.abs(got[:, fin] - ref[:, fin]).max(initial=0.0) <= (9 * spp + 8) * 2.0 ** -22
+    gv = var.cpu().numpy()
+    assert np.array_equal(np.isnan(gv), np.isnan(rvar))
+    assert np.abs(gv - rvar)[np.isfinite(rvar)].max(initial=0.0) <= (spp + 8) * 2.0 ** -22
+
+
+@pytest.mark.parametrize("size,shift", [((64, 5), 0), ((64, 5), 1), ((66, 5), 0), ((4, 3), 0), ((1, 1), 0)])
+def test_velocity_widths_and_alignments(size, shift):
+    """128-bit accesses where width and buffers allow them, else single values: the same bits."""
+    w, h = size
+    M = synth.orbit_camera(9, w, h)
+    world = synth.first_collision_world(w, h, synth.orbit_camera(10, w, h), seed=3, miss_frac=0.2)
+    buf, out = torch.empty(3 * h * w + 1, device="cuda"), torch.empty(2 * h * w + 1, device="cuda")
+    d, mot = buf[shift:shift + 3 * h * w].view(3, h, w), out[shift:shift + 2 * h * w].view(2, h, w)
+    d.copy_(torch.from_numpy(world))
+    W.wrls_velocity_from_world(d, M, mot)
+    got = mot.cpu().numpy()
+    ref = O.velocity(world, M.astype(np.float32).astype(np.float64))
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert np.nanmax(np.abs(got - ref), initial=0.0) <= 2e-3  # pixels, as at full HD
