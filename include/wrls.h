@@ -101,7 +101,7 @@ typedef struct wrls_params {
 
 /*
  * Extended path. Parameters with n_gbuf > 0, weight_mode 2 or reproj_filter 1 run on a
- * separate pair of kernels (one thread per pixel, binary32 state of 3d + d(d+1)/2 + 3 planes
+ * separate pair of kernels (binary32 state of 3d + d(d+1)/2 + 3 planes
  * per pixel: beta[c][a] at plane c*d + a, the upper triangle of P row by row, then z). They
  * need state_precision WRLS_STATE_F32 (WRLS_ERR_INVALID_ARG otherwise), take no blend tile
  * configuration other than 0, and are not accepted by the batched ticks.
@@ -201,9 +201,10 @@ wrls_status wrls_denoise_sequence_host(wrls_stream* s, const struct wrls_frame_i
 
 /* Not in the paper: CTAs per SM of the persistent blend kernels (blend configurations 4-9)
  * when they overlap an update in wrls_denoise_sequence: fewer leave the update room on every SM. 0 = as many
- * as fit; default 3 (measured at 1080p, binary32 state, configuration 9: 120.7 us per frame with
- * 3, 123.6 us with 2, about 235 us with 1; 16-bit state, configuration 8, whose CTAs are twice
- * as large: the same with 2 and 3). */
+ * as fit; default 4 (measured, us per frame with 2 / 3 / 4, binary32 state, configuration 9: 720p 61.1 /
+ * 58.3 / 57.3, 1080p 131.8 / 127.4 / 125.9, 2160p 523 / 502 / 496; 16-bit state, configuration 8, whose CTAs
+ * are twice as large and of which 2 fit: 1080p 129 with 1, 113 with 2).
+ */
 wrls_status wrls_stream_set_overlap(wrls_stream* s, int blend_ctas_per_sm);
 
 /* The next frame restarts every pixel (frame-0 behaviour: beta and P at their initial
@@ -271,8 +272,7 @@ uint64_t wrls_stream_frames(const wrls_stream* s);
  * launch (-1 for a configuration the state format does not offer) and *chosen (optional)
  * the selected configuration. Synchronises the stream. After wrls_stream_create the
  * configuration is, on images of at least 2^17 pixels (and 72 x 20), 9 for the binary32 state and 8
- * for the 16-bit formats, else
- * 2. wrls_batch_tick uses each stream's configuration; wrls_batch_tick_static uses a
+ * for the 16-bit formats, else 2. wrls_batch_tick uses each stream's configuration; wrls_batch_tick_static uses a
  * one-CTA-per-tile configuration of the same tile rows (2 for configurations 8 and 9).
  * Streams on the extended path have
  * one blend configuration: every time is reported as -1 and 0 is chosen, without a launch.

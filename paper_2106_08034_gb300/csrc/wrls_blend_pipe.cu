@@ -501,8 +501,9 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
     const int next = tile - (int)gridDim.x;
     if (next < 0) {
       pdl_next();
-    } else if (threadIdx.x == 0 && hint_ctas(kp) == 0) {
-      // the next window into L2 (beside an update, whose traffic it delays, this costs 1 % at 2160p)
+    } else if (threadIdx.x == 0 && hint_pdl(kp)) {
+      // per-frame calls: the next window into L2 (beside an update, whose traffic it delays, this
+      // costs 1 % at 2160p)
       const int x = (next % tiles_x) * TW2 - 4, y = (next / tiles_x) * TH - 2;
       tma_prefetch_3d(mz, x, y, kZ);
       tma_prefetch_3d(mb, x, y, 0);

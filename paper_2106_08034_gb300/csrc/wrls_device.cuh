@@ -657,7 +657,6 @@ struct PairTaps {
   float2 w[4];
 };
 
-template <int TAPS>
 __device__ __forceinline__ float2 tap_add(int t, float2 w, float2 v, float2 acc) {
   return t == 0 ? f2mul(w, v) : f2fma(w, v, acc);
 }
@@ -685,9 +684,9 @@ struct PairState<State16<T>> {
       tap(s, 11, t.o0[k], t.o1[k], z0, z1);
       const uint32_t u0 = s.word(12, t.o0[k]), u1 = s.word(12, t.o1[k]);
       const float2 z2 = make_float2(SV::unpack(u0).x, SV::unpack(u1).x);
-      v[0] = tap_add<TAPS>(k, t.w[k], z0, v[0]);
-      v[1] = tap_add<TAPS>(k, t.w[k], z1, v[1]);
-      v[2] = tap_add<TAPS>(k, t.w[k], z2, v[2]);
+      v[0] = tap_add(k, t.w[k], z0, v[0]);
+      v[1] = tap_add(k, t.w[k], z1, v[1]);
+      v[2] = tap_add(k, t.w[k], z2, v[2]);
       q[k] = f2mul(t.w[k], make_float2(SV::scale_of(u0), SV::scale_of(u1)));
     }
   }
@@ -700,16 +699,16 @@ struct PairState<State16<T>> {
       for (int w = 0; w < 5; ++w) tap(s, 6 + w, t.o0[k], t.o1[k], l[2 * w], l[2 * w + 1]);
       // P / s = L L^T of the tap, rows of L: l[0] | l[1] l[4] | l[2] l[5] l[7] | l[3] l[6] l[8] l[9]
       const float2 w = q[k];
-      P[0] = tap_add<TAPS>(k, w, f2mul(l[0], l[0]), P[0]);
-      P[1] = tap_add<TAPS>(k, w, f2mul(l[1], l[0]), P[1]);
-      P[2] = tap_add<TAPS>(k, w, f2mul(l[2], l[0]), P[2]);
-      P[3] = tap_add<TAPS>(k, w, f2mul(l[3], l[0]), P[3]);
-      P[4] = tap_add<TAPS>(k, w, f2fma(l[4], l[4], f2mul(l[1], l[1])), P[4]);
-      P[5] = tap_add<TAPS>(k, w, f2fma(l[5], l[4], f2mul(l[2], l[1])), P[5]);
-      P[6] = tap_add<TAPS>(k, w, f2fma(l[6], l[4], f2mul(l[3], l[1])), P[6]);
-      P[7] = tap_add<TAPS>(k, w, f2fma(l[7], l[7], f2fma(l[5], l[5], f2mul(l[2], l[2]))), P[7]);
-      P[8] = tap_add<TAPS>(k, w, f2fma(l[8], l[7], f2fma(l[6], l[5], f2mul(l[3], l[2]))), P[8]);
-      P[9] = tap_add<TAPS>(k, w, f2fma(l[9], l[9], f2fma(l[8], l[8], f2fma(l[6], l[6], f2mul(l[3], l[3])))), P[9]);
+      P[0] = tap_add(k, w, f2mul(l[0], l[0]), P[0]);
+      P[1] = tap_add(k, w, f2mul(l[1], l[0]), P[1]);
+      P[2] = tap_add(k, w, f2mul(l[2], l[0]), P[2]);
+      P[3] = tap_add(k, w, f2mul(l[3], l[0]), P[3]);
+      P[4] = tap_add(k, w, f2fma(l[4], l[4], f2mul(l[1], l[1])), P[4]);
+      P[5] = tap_add(k, w, f2fma(l[5], l[4], f2mul(l[2], l[1])), P[5]);
+      P[6] = tap_add(k, w, f2fma(l[6], l[4], f2mul(l[3], l[1])), P[6]);
+      P[7] = tap_add(k, w, f2fma(l[7], l[7], f2fma(l[5], l[5], f2mul(l[2], l[2]))), P[7]);
+      P[8] = tap_add(k, w, f2fma(l[8], l[7], f2fma(l[6], l[5], f2mul(l[3], l[2]))), P[8]);
+      P[9] = tap_add(k, w, f2fma(l[9], l[9], f2fma(l[8], l[8], f2fma(l[6], l[6], f2mul(l[3], l[3])))), P[9]);
     }
   }
   template <int TAPS, class Src>
@@ -720,7 +719,7 @@ struct PairState<State16<T>> {
       tap(s, 2 * c, t.o0[k], t.o1[k], v[0], v[1]);
       tap(s, 2 * c + 1, t.o0[k], t.o1[k], v[2], v[3]);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) b[a] = tap_add<TAPS>(k, t.w[k], v[a], b[a]);
+      for (int a = 0; a < 4; ++a) b[a] = tap_add(k, t.w[k], v[a], b[a]);
     }
   }
   static __device__ __forceinline__ void put(const SV& n, uint32_t i, uint32_t i1, int k, uint32_t u0, uint32_t u1, bool in0, bool in1) {
