@@ -86,6 +86,30 @@ __device__ __forceinline__ float blend_rk(float z0, float z1, float z2, float ep
 __device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Loads of global memory in the kernels that call pdl_wait(). What they read (state planes, frame
+// inputs) may still be written by the kernel before while they are already resident. __ldg, and plain
+// reads through a const __restrict__ parameter, promise that the data does not change during the
+// kernel's life, so the compiler may place them ahead of the wait and the hardware may serve them from
+// a cache that is not kept coherent. These are ordinary loads, volatile so that they stay behind the
+// wait, after which everything the kernel before wrote is visible to them.
+__device__ __forceinline__ float ld_global(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ float4 ld_global(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+
 // ---- packed binary32 pairs (sm_100 family: one instruction for two lanes' worth) ----------
 // Each component is rounded as the scalar operation would be (round to nearest even, no
 // flush), so a packed loop gives bitwise the results of its scalar form.
@@ -237,13 +261,13 @@ struct StateF32 {
   int pitch;
   __device__ __forceinline__ void load(size_t idx, float v[kNState]) const {
 #pragma unroll
-    for (int p = 0; p < kNState; ++p) v[p] = __ldg(base + p * plane_stride + idx);
+    for (int p = 0; p < kNState; ++p) v[p] = ld_global(base + p * plane_stride + idx);
   }
   __device__ __forceinline__ void load_beta_z(size_t idx, float b[12], float z[3]) const {
 #pragma unroll
-    for (int p = 0; p < 12; ++p) b[p] = __ldg(base + p * plane_stride + idx);
+    for (int p = 0; p < 12; ++p) b[p] = ld_global(base + p * plane_stride + idx);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) z[c] = __ldg(base + (kZ + c) * plane_stride + idx);
+    for (int c = 0; c < 3; ++c) z[c] = ld_global(base + (kZ + c) * plane_stride + idx);
   }
   // idx < 2^32: each plane's base is uniform over the warp and the pixel offset 32-bit
   __device__ __forceinline__ void store(size_t idx, const float v[kNState]) const {
@@ -354,7 +378,7 @@ struct State16 {
     uint32_t w[kPlanes];
     float s;
 #pragma unroll
-    for (int k = 0; k < kPlanes; ++k) w[k] = __ldg(base + k * plane_stride + idx);
+    for (int k = 0; k < kPlanes; ++k) w[k] = ld_global(base + k * plane_stride + idx);
     decode(w, v, s);
 #pragma unroll
     for (int p = kP; p < kZ; ++p) v[p] *= s;
@@ -362,14 +386,14 @@ struct State16 {
   __device__ __forceinline__ void load_beta_z(size_t idx, float b[12], float z[3]) const {
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      const float2 f = unpack(__ldg(base + k * plane_stride + idx));
+      const float2 f = unpack(ld_global(base + k * plane_stride + idx));
       b[2 * k] = f.x;
       b[2 * k + 1] = f.y;
     }
-    const float2 z01 = unpack(__ldg(base + 11 * plane_stride + idx));
+    const float2 z01 = unpack(ld_global(base + 11 * plane_stride + idx));
     z[0] = z01.x;
     z[1] = z01.y;
-    z[2] = unpack(__ldg(base + 12 * plane_stride + idx)).x;
+    z[2] = unpack(ld_global(base + 12 * plane_stride + idx)).x;
   }
   __device__ __forceinline__ void store(size_t idx, const float v[kNState]) const {
     const int e = scale_exponent(fmaxf(fmaxf(v[kP + 0], v[kP + 4]), fmaxf(v[kP + 7], v[kP + 9])));
@@ -643,7 +667,7 @@ struct GlobalTaps {
   const uint32_t* base;
   size_t plane_stride;
   __device__ __forceinline__ uint32_t word(int p, int i) const {
-    return __ldg(base + (size_t)p * plane_stride + (uint32_t)i);
+    return ld_global(base + (size_t)p * plane_stride + (uint32_t)i);
   }
 };
 

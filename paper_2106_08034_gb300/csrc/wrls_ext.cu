@@ -67,7 +67,7 @@ struct ExtStaged {
 struct ExtGlobal {
   const float* base;
   size_t ps;
-  __device__ __forceinline__ float at(int, int, int p, int o) const { return __ldg(base + (size_t)p * ps + (uint32_t)o); }
+  __device__ __forceinline__ float at(int, int, int p, int o) const { return ld_global(base + (size_t)p * ps + (uint32_t)o); }
 };
 
 struct ExtTaps {
@@ -98,8 +98,8 @@ __device__ __forceinline__ void ext_gather(const Src& s, const ExtTaps& t, int o
 template <int D, bool F, int TAPS, class Src, class Ready>
 __device__ __forceinline__ void ext_update_pixel(const ExtParams& ep, const Src& src, const ExtTaps& t, const bool valid,
                                                  const float I[3], const bool missing, const float lo[3],
-                                                 const float hi[3], const float* __restrict__ var,
-                                                 const float* __restrict__ gbuf, const size_t npix, const size_t j,
+                                                 const float hi[3], const float* var,
+                                                 const float* gbuf, const size_t npix, const size_t j,
                                                  float* __restrict__ dst, const size_t ps, const bool inside,
                                                  Ready&& ready) {
   using L = ExtDim<D, F>;
@@ -128,7 +128,7 @@ __device__ __forceinline__ void ext_update_pixel(const ExtParams& ep, const Src&
   bool g_ok = true;
 #pragma unroll
   for (int i = 0; i < L::kG; ++i) {
-    const float g = inside ? __ldg(gbuf + (size_t)i * npix + j) : 0.0f;
+    const float g = inside ? ld_global(gbuf + (size_t)i * npix + j) : 0.0f;
     const bool f = isfinite(g);
     p[L::kG0 + i] = f ? g : 0.0f;
     g_ok = g_ok && f;
@@ -144,7 +144,7 @@ __device__ __forceinline__ void ext_update_pixel(const ExtParams& ep, const Src&
     const float nz = sqrtf(z[0] * z[0] + z[1] * z[1] + z[2] * z[2]);
     const float m = fminf(nI, nz) + kp.eps;
     if (kp.weight_mode == 2) {
-      const float v = inside ? __ldg(var + j) : 0.0f;
+      const float v = inside ? ld_global(var + j) : 0.0f;
       w = (isfinite(v) && v >= 0.0f) ? ex2_approx(-(v / (m * m)) * ep.wv_k) : 0.0f;
     } else {
       const float d0 = I[0] - z[0], d1 = I[1] - z[1], d2 = I[2] - z[2];
@@ -246,9 +246,9 @@ __device__ __forceinline__ void ext_update_pixel(const ExtParams& ep, const Src&
 template <int D, bool F>
 __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
     k_update_ext(const ExtParams ep, const int W, const int H, const int reset, const int stage_ok,
-                 const float* __restrict__ prev, float* __restrict__ next, const int pitch, const size_t ps,
-                 const __grid_constant__ ExtStageMaps maps, const float* __restrict__ rad,
-                 const float* __restrict__ mot, const float* __restrict__ var, const float* __restrict__ gbuf, int* err) {
+                 const float* prev, float* __restrict__ next, const int pitch, const size_t ps,
+                 const __grid_constant__ ExtStageMaps maps, const float* rad,
+                 const float* mot, const float* var, const float* gbuf, int* err) {
   using L = ExtDim<D, F>;
   using S = ExtStage<D, F>;
   const KParams& kp = ep.kp;
@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
   float qx = 0.0f, qy = 0.0f;
   bool valid = false;
   if (inside) {
-    qx = (float)x + __ldg(mot + j);
-    qy = (float)y + __ldg(mot + npix + j);
+    qx = (float)x + ld_global(mot + j);
+    qy = (float)y + ld_global(mot + npix + j);
     valid = !reset && qx >= 0.0f && qx <= (float)(W - 1) && qy >= 0.0f && qy <= (float)(H - 1);
   }
   const bool nearest = ep.reproj_filter == 1;
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
   bool missing = true;
   if (inside) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) I[c] = __ldg(rad + c * npix + j);
+    for (int c = 0; c < 3; ++c) I[c] = ld_global(rad + c * npix + j);
     missing = !finite3(I);
     if (kp.clamp_mode == 0) {
       // Psi = clamp to the 3x3 min/max of the finite samples: a neighbour outside the image is
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
 #pragma unroll
         for (int dx = -1; dx <= 1; ++dx) {
           const size_t jj = (size_t)min(max(y + dy, 0), H - 1) * W + min(max(x + dx, 0), W - 1);
-          const float In[3] = {__ldg(rad + jj), __ldg(rad + npix + jj), __ldg(rad + 2 * npix + jj)};
+          const float In[3] = {ld_global(rad + jj), ld_global(rad + npix + jj), ld_global(rad + 2 * npix + jj)};
           const bool fin = finite3(In);
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
@@ -387,19 +387,19 @@ constexpr float kExtFarZ = 1e18f;  // feature of an out-of-image neighbour: its 
 constexpr int kExtBlendRows = 2;
 
 template <int D, bool F>
-__device__ __forceinline__ void ext_predictor_g(const float* __restrict__ gbuf, size_t npix, size_t j, float p[D]) {
+__device__ __forceinline__ void ext_predictor_g(const float* gbuf, size_t npix, size_t j, float p[D]) {
   using L = ExtDim<D, F>;
 #pragma unroll
   for (int i = 0; i < L::kG; ++i) {
-    const float g = __ldg(gbuf + (size_t)i * npix + j);
+    const float g = ld_global(gbuf + (size_t)i * npix + j);
     p[L::kG0 + i] = isfinite(g) ? g : 0.0f;
   }
 }
 
 template <int D, bool F>
 __global__ void __launch_bounds__(kExtTW * kExtTH / kExtBlendRows)
-    k_blend_ext(const ExtParams ep, const int W, const int H, const float* __restrict__ cur, const int pitch,
-                const size_t ps, const float* __restrict__ gbuf, float* __restrict__ out) {
+    k_blend_ext(const ExtParams ep, const int W, const int H, const float* cur, const int pitch,
+                const size_t ps, const float* gbuf, float* __restrict__ out) {
   using L = ExtDim<D, F>;
   constexpr int NPL = 3 * D + 4;  // beta planes, z (3), range factor
   constexpr int NT = kExtTW * kExtTH / kExtBlendRows;
@@ -414,9 +414,9 @@ __global__ void __launch_bounds__(kExtTW * kExtTH / kExtBlendRows)
     if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
       const float* src = cur + (size_t)gy * pitch + gx;
 #pragma unroll
-      for (int a = 0; a < 3 * D; ++a) sm[a * kExtSP + e] = __ldg(src + (L::kBeta + a) * ps);
-      const float z0 = __ldg(src + (L::kZ + 0) * ps), z1 = __ldg(src + (L::kZ + 1) * ps),
-                  z2 = __ldg(src + (L::kZ + 2) * ps);
+      for (int a = 0; a < 3 * D; ++a) sm[a * kExtSP + e] = ld_global(src + (L::kBeta + a) * ps);
+      const float z0 = ld_global(src + (L::kZ + 0) * ps), z1 = ld_global(src + (L::kZ + 1) * ps),
+                  z2 = ld_global(src + (L::kZ + 2) * ps);
       sm[(3 * D + 0) * kExtSP + e] = z0;
       sm[(3 * D + 1) * kExtSP + e] = z1;
       sm[(3 * D + 2) * kExtSP + e] = z2;
@@ -541,7 +541,7 @@ constexpr int ext2_smem_bytes() { return (3 * D + 4) * kExt2Plane * 4 + 128; }
 template <int D, bool F>
 __global__ void __launch_bounds__(128)
     k_blend_ext2(const ExtParams ep, const int W, const int H, const __grid_constant__ ExtMaps maps,
-                 const float* __restrict__ gbuf, float* __restrict__ out, int* err) {
+                 const float* gbuf, float* __restrict__ out, int* err) {
   using L = ExtDim<D, F>;
   constexpr int P = kExt2Plane, SW = kBlendBoxW2, Z = 3 * D;  // window planes: beta, z (3), range factor
   extern __shared__ unsigned char dsmem[];
@@ -569,8 +569,8 @@ __global__ void __launch_bounds__(128)
     for (int a = 0; a < L::kG; ++a) {
       float2 g = make_float2(0.0f, 0.0f);
       const float* s = gbuf + (size_t)a * npix + (size_t)(y0 + i) * W + x;
-      if (y0 + i < H && x < W) g.x = __ldg(s);
-      if (y0 + i < H && x + 1 < W) g.y = __ldg(s + 1);
+      if (y0 + i < H && x < W) g.x = ld_global(s);
+      if (y0 + i < H && x + 1 < W) g.y = ld_global(s + 1);
       pi[i][L::kG0 + a] = make_float2(isfinite(g.x) ? g.x : 0.0f, isfinite(g.y) ? g.y : 0.0f);
     }
   __syncthreads();  // the barriers are initialised

@@ -11,7 +11,7 @@ template <class SV>
 __global__ void __launch_bounds__(update_threads<SV>(), update_min_ctas<SV>())
     k_update(const KParams kp, const int W, const int H, const int reset, const int stage_ok,
              const SV prev, const SV next, const __grid_constant__ StageMaps maps,
-             const float* __restrict__ rad, const float* __restrict__ mot, int* err) {
+             const float* rad, const float* mot, int* err) {
   extern __shared__ unsigned char dsmem[];
   __shared__ alignas(8) uint64_t bar;
   UpdateSmem<SV>& sm = *reinterpret_cast<UpdateSmem<SV>*>(align128(dsmem));
@@ -45,14 +45,14 @@ __global__ void k_read_state(const int W, const int H, const SV cur, float* __re
 
 // Inverse of k_read_state: binary32 planes in, the state copy encoded in its format.
 template <class SV>
-__global__ void k_write_state(const int W, const int H, const SV cur, const float* __restrict__ src) {
+__global__ void k_write_state(const int W, const int H, const SV cur, const float* src) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   pdl_wait();
   if (x >= W || y >= H) return;
   const size_t npix = (size_t)W * H, j = (size_t)y * W + x;
   float v[kNState];
 #pragma unroll
-  for (int p = 0; p < kNState; ++p) v[p] = src[p * npix + j];
+  for (int p = 0; p < kNState; ++p) v[p] = ld_global(src + p * npix + j);
   pdl_next();
   cur.store((size_t)y * cur.pitch + x, v);
 }

@@ -47,8 +47,8 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* 
                                            const KParams& kp, const int W, const int H,
                                            const bool reset, const bool stage_ok, const StateF32& prev,
                                            const StateF32& next, const StageMaps* maps,
-                                           const float* __restrict__ rad,
-                                           const float* __restrict__ mot, const int bx0,
+                                           const float* rad,
+                                           const float* mot, const int bx0,
                                            const int by0) {
   const int tx = threadIdx.x % kTW, ty = threadIdx.x / kTW;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -62,8 +62,8 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* 
   float qx = 0.0f, qy = 0.0f;
   bool valid = false;
   if (inside) {
-    qx = (float)x + __ldg(mot + j);
-    qy = (float)y + __ldg(mot + npix + j);
+    qx = (float)x + ld_global(mot + j);
+    qy = (float)y + ld_global(mot + npix + j);
     valid = !reset && qx >= 0.0f && qx <= (float)(W - 1) && qy >= 0.0f && qy <= (float)(H - 1);
   }
   int lo_x = 0x7fffffff, hi_x = -1, lo_y = 0x7fffffff, hi_y = -1;
@@ -115,9 +115,9 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* 
     float r = nan, g = nan, b = nan;
     if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
       const size_t jj = (size_t)gy * W + gx;
-      r = __ldg(rad + jj);
-      g = __ldg(rad + npix + jj);
-      b = __ldg(rad + 2 * npix + jj);
+      r = ld_global(rad + jj);
+      g = ld_global(rad + npix + jj);
+      b = ld_global(rad + 2 * npix + jj);
       if (!(isfinite(r) && isfinite(g) && isfinite(b))) r = g = b = nan;
     }
     sm.rad[0][ly][lx] = r;
@@ -171,14 +171,14 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* 
 // the image give (NaN, NaN, NaN): fminf/fmaxf ignore NaN operands, so the clamp box skips them
 // without a test per neighbour.
 struct Rgb { float r, g, b; };
-__device__ __forceinline__ Rgb load_radiance(const float* __restrict__ rad, size_t npix, int gx, int gy, int W, int H) {
+__device__ __forceinline__ Rgb load_radiance(const float* rad, size_t npix, int gx, int gy, int W, int H) {
   const float nan = __int_as_float(0x7fc00000);
   Rgb v{nan, nan, nan};
   if ((unsigned)gx < (unsigned)W && (unsigned)gy < (unsigned)H) {
     const float* p = rad + (size_t)gy * W + gx;
-    v.r = __ldg(p);
-    v.g = __ldg(p + npix);
-    v.b = __ldg(p + 2 * npix);
+    v.r = ld_global(p);
+    v.g = ld_global(p + npix);
+    v.b = ld_global(p + 2 * npix);
     // 0 * v is NaN for a non-finite v
     const float t = fmaf(v.b, 0.0f, fmaf(v.g, 0.0f, v.r * 0.0f));
     if (t != t) v.r = v.g = v.b = nan;
@@ -194,8 +194,8 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, u
                                            const KParams& kp, const int W, const int H,
                                            const bool reset, const bool stage_ok, const SV& prev,
                                            const SV& next, const StageMaps* maps,
-                                           const float* __restrict__ rad,
-                                           const float* __restrict__ mot, const int bx0,
+                                           const float* rad,
+                                           const float* mot, const int bx0,
                                            const int by0) {
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;  // lane, warp: the tile row(s) of a warp
   const size_t npix = (size_t)W * H;
@@ -207,8 +207,8 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, u
   {
     const float* m = mot + (size_t)ya * W + xa;
     const size_t step = (size_t)kPairY * W;
-    if (in0) { qx0 = __ldg(m); qy0 = __ldg(m + npix); }
-    if (in1) { qx1 = __ldg(m + step); qy1 = __ldg(m + step + npix); }
+    if (in0) { qx0 = ld_global(m); qy0 = ld_global(m + npix); }
+    if (in1) { qx1 = ld_global(m + step); qy1 = ld_global(m + step + npix); }
   }
   qx0 += (float)xa; qy0 += (float)ya;
   qx1 += (float)xb; qy1 += (float)yb;

@@ -41,7 +41,7 @@ constexpr int kRecChunk = 2;
 
 template <bool VAR>
 __global__ void __launch_bounds__(kRecThreads, 12)
-    k_reconstruct(const ReconArgs a, const int W, const int H, const int spp, const float* __restrict__ smp,
+    k_reconstruct(const ReconArgs a, const int W, const int H, const int spp, const float* smp,
                   float* __restrict__ out, float* __restrict__ var) {
   __shared__ float sm[kRecChunk][5][kRecSP];
   const int bx0 = blockIdx.x * kRecTW, by0 = blockIdx.y * kRecTH;
@@ -62,11 +62,11 @@ __global__ void __launch_bounds__(kRecThreads, 12)
     float r = 0.0f, g = 0.0f, b = 0.0f, ox = INFINITY, oy = INFINITY;
     if ((unsigned)gx < (unsigned)W && (unsigned)gy < (unsigned)H) {
       const float* base = smp + (size_t)s * 5 * np + (size_t)gy * W + gx;
-      r = __ldg(base);
-      g = __ldg(base + np);
-      b = __ldg(base + 2 * np);
-      ox = __ldg(base + 3 * np);
-      oy = __ldg(base + 4 * np);
+      r = ld_global(base);
+      g = ld_global(base + np);
+      b = ld_global(base + 2 * np);
+      ox = ld_global(base + 3 * np);
+      oy = ld_global(base + 4 * np);
       // 0 * v is NaN for a non-finite v
       const float t = fmaf(oy, 0.0f, fmaf(ox, 0.0f, fmaf(b, 0.0f, fmaf(g, 0.0f, r * 0.0f))));
       if (t != t) {
@@ -191,7 +191,7 @@ struct Mat4 {
 // next launch in early: its many small CTAs would contend (12.4 -> 18.8 us).
 template <int V>
 __global__ void k_velocity(const Mat4 M, const int W, const int H, const int miss_policy,
-                           const float* __restrict__ world, float* __restrict__ mot) {
+                           const float* world, float* __restrict__ mot) {
   const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * V, y = blockIdx.y;
   pdl_wait();
   if (x0 >= W || y >= H) return;
@@ -200,13 +200,13 @@ __global__ void k_velocity(const Mat4 M, const int W, const int H, const int mis
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     if (V == 4) {
-      const float4 t = __ldg(reinterpret_cast<const float4*>(world + c * np + j));
+      const float4 t = ld_global(reinterpret_cast<const float4*>(world + c * np + j));
       p[c][0] = t.x;
       p[c][V > 1 ? 1 : 0] = t.y;
       p[c][V > 2 ? 2 : 0] = t.z;
       p[c][V > 3 ? 3 : 0] = t.w;
     } else {
-      p[c][0] = __ldg(world + c * np + j);
+      p[c][0] = ld_global(world + c * np + j);
     }
   }
   if (V == 4) pdl_next();
