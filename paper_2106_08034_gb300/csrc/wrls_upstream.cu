@@ -288,7 +288,9 @@ wrls_status wrls_reconstruct(int width, int height, int spp, const float* sample
     return WRLS_ERR_INVALID_ARG;
   }
   ReconArgs a;
-  a.k2 = (float)(1.4426950408889634 / (2.0 * (double)p->sigma * (double)p->sigma));
+  // k2 stays above 0 (sigma up to infinity: a box filter, weight 2^-0 = 1 within the support), so that
+  // the infinite offset of a missing sample or of one outside the image gives 2^-inf = 0, not inf * 0 = NaN
+  a.k2 = fmaxf((float)(1.4426950408889634 / (2.0 * (double)p->sigma * (double)p->sigma)), 1.17549435e-38f);
   a.radius = p->radius;
   const dim3 grid((width + kRecTW - 1) / kRecTW, (height + kRecTH - 1) / kRecTH);
   cudaStream_t cs = (cudaStream_t)cuda_stream;

@@ -151,3 +151,25 @@ def test_velocity_widths_and_alignments(size, shift):
     ref = O.velocity(world, M.astype(np.float32).astype(np.float64))
     assert np.array_equal(np.isnan(got), np.isnan(ref))
     assert np.nanmax(np.abs(got - ref), initial=0.0) <= 2e-3  # pixels, as at full HD
+
+
+# sigma beyond 3e22 leaves a binary32 exponent factor of 0; infinity asks for a box filter
+@pytest.mark.parametrize("sigma", [1e19, 1e23, float("inf")])
+@pytest.mark.parametrize("size", [(61, 23), (33, 9)])
+@pytest.mark.parametrize("radius,far", [(1.5, False), (1.2, True)])
+def test_reconstruction_with_a_very_wide_filter(sigma, size, radius, far):
+    """Samples outside the image or the support and missing samples still have weight 0."""
+    w, h = size
+    gen = torch.Generator().manual_seed(w + h)
+    smp = torch.rand(2, 5, h, w, generator=gen)
+    smp[:, 3:] -= 0.5
+    if far:
+        smp[:, 3:][torch.rand(2, 2, h, w, generator=gen) < 0.1] *= 2.5
+    smp[:, 0][torch.rand(2, h, w, generator=gen) < 0.1] = float("nan")
+    rad, var = torch.empty(3, h, w, device="cuda"), torch.empty(h, w, device="cuda")
+    W.wrls_reconstruct(smp.cuda(), rad, var, W.wrls_recon_params_default(sigma=sigma, radius=radius))
+    ref, rvar = O.reconstruct(smp.numpy(), sigma=float(np.float32(sigma)), radius=float(np.float32(radius)))
+    got, gv = rad.cpu().numpy(), var.cpu().numpy()
+    assert np.isfinite(ref).all() and np.isfinite(got).all()
+    assert np.abs(got - ref).max() <= (9 * 2 + 8) * 2.0 ** -22  # as in the tile-edge test
+    assert np.array_equal(np.isnan(gv), np.isnan(rvar))
