@@ -188,15 +188,10 @@ template <int TH, int R, int MODE, int NBUF>
 static cudaError_t launch_tma_cfg(const KParams& kp, const StateDesc& cur, float* out, int* err, cudaStream_t cs) {
   constexpr int bytes = TmaBlendGeom<TH>::smem_bytes(NBUF);
   constexpr int nt = kTW * TH / R;
-  static int per_sm = 0;  // per instantiation
-  if (!per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_blend_tma<TH, R, MODE, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_tma<TH, R, MODE, NBUF>, nt, bytes);
-    if (e != cudaSuccess) return e;
-    per_sm = occ > 0 ? occ : 1;
-  }
+  static KernelSetup setup;  // per instantiation
+  int per_sm = 1;
+  const cudaError_t e = setup(k_blend_tma<TH, R, MODE, NBUF>, nt, bytes, &per_sm);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -561,15 +556,10 @@ template <int TH, int R, int MODE>
 static cudaError_t launch_tma2_cfg(const KParams& kp, const StateDesc& cur, float* out, int* err, cudaStream_t cs) {
   constexpr int bytes = TmaBlend2Geom<TH>::kSmemBytes;
   constexpr int nt = kTW * TH / R;
-  static int per_sm = 0;  // per instantiation
-  if (!per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_blend_tma2<TH, R, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_tma2<TH, R, MODE>, nt, bytes);
-    if (e != cudaSuccess) return e;
-    per_sm = occ > 0 ? occ : 1;
-  }
+  static KernelSetup setup;  // per instantiation
+  int per_sm = 1;
+  const cudaError_t e = setup(k_blend_tma2<TH, R, MODE>, nt, bytes, &per_sm);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -731,15 +721,10 @@ template <int TH, int R, int MODE, typename T>
 static cudaError_t launch_tma2h_cfg(const KParams& kp, const StateDesc& cur, float* out, int* err, cudaStream_t cs) {
   constexpr int bytes = TmaBlend2hGeom<TH>::kSmemBytes;
   constexpr int nt = kTW * TH / R;
-  static int per_sm = 0;  // per instantiation
-  if (!per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_blend_tma2h<TH, R, MODE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_tma2h<TH, R, MODE, T>, nt, bytes);
-    if (e != cudaSuccess) return e;
-    per_sm = occ > 0 ? occ : 1;
-  }
+  static KernelSetup setup;  // per instantiation
+  int per_sm = 1;
+  const cudaError_t e = setup(k_blend_tma2h<TH, R, MODE, T>, nt, bytes, &per_sm);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

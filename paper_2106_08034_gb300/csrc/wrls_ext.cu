@@ -701,12 +701,9 @@ static cudaError_t launch_ext_t(const ExtParams& ep, const StateDesc& prev, cons
                                 const float* rad, const float* mot, const float* var, const float* gbuf, int* err,
                                 cudaStream_t cs) {
   constexpr int bytes = ExtStage<D, F>::kSmemBytes;
-  static bool attr_set = false;  // per instantiation
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_update_ext<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static KernelSetup setup;  // per instantiation
+  const cudaError_t e = setup(k_update_ext<D, F>, kExtTW * kExtTH, bytes);
+  if (e != cudaSuccess) return e;
   const dim3 grid((prev.W + kExtTW - 1) / kExtTW, (prev.H + kExtTH - 1) / kExtTH);
   return launch_kernel(k_update_ext<D, F>, grid, kExtTW * kExtTH, bytes, cs, hint_pdl(ep.kp), ep, prev.W, prev.H, reset ? 1 : 0,
                        prev.stage_ok ? 1 : 0, (const float*)prev.base, (float*)next.base, prev.pitch, prev.plane_stride,
@@ -718,12 +715,9 @@ static cudaError_t launch_ext_blend_t(const ExtParams& ep, const StateDesc& cur,
                                       int* err, cudaStream_t cs) {
   if (ep.kp.blend_mode == 0 && cur.ext_tma_ok) {
     constexpr int bytes = ext2_smem_bytes<D>();
-    static bool attr_set = false;  // per instantiation
-    if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(k_blend_ext2<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-      if (e != cudaSuccess) return e;
-      attr_set = true;
-    }
+    static KernelSetup setup;  // per instantiation
+    const cudaError_t e = setup(k_blend_ext2<D, F>, 128, bytes);
+    if (e != cudaSuccess) return e;
     const dim3 grid((cur.W + kExt2W - 1) / kExt2W, (cur.H + kExt2H - 1) / kExt2H);
     return launch_kernel(k_blend_ext2<D, F>, grid, 128, bytes, cs, hint_pdl(ep.kp), ep, cur.W, cur.H, cur.emaps, gbuf, out, err);
   }

@@ -62,12 +62,9 @@ static cudaError_t launch_update_t(const KParams& kp, const StateDesc& prev, con
                                   bool reset, const float* rad, const float* mot, int* err,
                                   cudaStream_t cs) {
   constexpr int bytes = update_smem_bytes<SV>();
-  static bool attr_set = false;  // per instantiation
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_update<SV>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static KernelSetup setup;  // per instantiation
+  const cudaError_t e = setup(k_update<SV>, update_threads<SV>(), bytes);
+  if (e != cudaSuccess) return e;
   const dim3 grid((prev.W + kTW - 1) / kTW, (prev.H + kTH - 1) / kTH);
   return launch_kernel(k_update<SV>, grid, update_threads<SV>(), bytes, cs, hint_pdl(kp), kp, prev.W, prev.H, reset ? 1 : 0,
                        prev.stage_ok ? 1 : 0, pv, nx, prev.maps, rad, mot, err);
@@ -87,13 +84,9 @@ template <class SV, int TH, int R, int MODE>
 static cudaError_t launch_blend_cfg(const KParams& kp, const SV& cur, int W, int H, float* out,
                                     cudaStream_t cs) {
   constexpr int bytes = BlendGeom<TH>::kSmemBytes;
-  static bool attr_set = false;  // per instantiation
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_blend<SV, TH, R, MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static KernelSetup setup;  // per instantiation
+  const cudaError_t e = setup(k_blend<SV, TH, R, MODE>, kTW * TH / R, bytes);
+  if (e != cudaSuccess) return e;
   const dim3 grid((W + kTW - 1) / kTW, (H + TH - 1) / TH);
   return launch_kernel(k_blend<SV, TH, R, MODE>, grid, kTW * TH / R, bytes, cs, hint_pdl(kp), kp, W, H, cur, out);
 }

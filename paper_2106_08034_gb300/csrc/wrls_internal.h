@@ -4,6 +4,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/wrls.h"
@@ -99,6 +101,32 @@ cudaError_t launch_read_state(const StateDesc& cur, float* dst, cudaStream_t cs)
 cudaError_t launch_write_state(const StateDesc& cur, const float* src, cudaStream_t cs);
 
 void set_error(const char* fmt, ...);
+
+// Set-up of one kernel for its launches: its opt-in to large dynamic shared memory and the CTAs of it
+// that fit an SM. Both belong to a device, so they are done on the first launch on each (a static
+// KernelSetup per kernel instantiation); devices beyond kDevices are set up on every launch.
+struct KernelSetup {
+  static constexpr int kDevices = 64;
+  std::atomic<int> per_sm[kDevices] = {};  // 0: not set up on that device
+
+  template <class K>
+  cudaError_t operator()(K* kernel, int threads, int smem_bytes, int* ctas_per_sm = nullptr) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool keep = dev >= 0 && dev < kDevices;
+    int occ = keep ? per_sm[dev].load(std::memory_order_acquire) : 0;
+    if (!occ) {
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem_bytes);
+      if (e != cudaSuccess) return e;
+      if (occ < 1) occ = 1;
+      if (keep) per_sm[dev].store(occ, std::memory_order_release);
+    }
+    if (ctas_per_sm) *ctas_per_sm = occ;
+    return cudaSuccess;
+  }
+};
 
 // Whether a kernel on `cs` may be launched with that attribute: not under stream capture.
 inline bool pdl_allowed(cudaStream_t cs) {

@@ -1,0 +1,83 @@
+"""Host side of the launches, followed with a stand-in CUDA runtime of two devices (no GPU needed)."""
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2106_08034_gb300 import build as B
+from paper_2106_08034_gb300 import wrls as W
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+WIDTH, HEIGHT = 512, 300  # above the size where the two-wide blend becomes the default
+PLANE = WIDTH * HEIGHT
+BUF = np.zeros(32 * PLANE, np.float32)
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    """The library's objects linked with fake_cudart.cpp in place of the CUDA runtime."""
+    B.build()
+    sources = glob.glob(os.path.join(B.CSRC, "*.cu"))
+    objs = [os.path.join(B.OUT_DIR, os.path.basename(s)[:-3] + ".o") for s in sorted(sources)]
+    if not all(os.path.exists(o) for o in objs):
+        B.build(force=True)
+    so = str(tmp_path_factory.mktemp("fake") / "libwrls_fake.so")
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    # -Bsymbolic: the library's calls reach the stand-in even where a CUDA runtime is loaded already
+    cmd = ["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", include, "-o", so,
+           os.path.join(HERE, "fake_cudart.cpp")] + objs
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
+    saved = W._lib, W.LIB_PATH
+    W._lib, W.LIB_PATH = None, so
+    try:
+        yield W.lib()
+    finally:
+        W._lib, W.LIB_PATH = saved
+
+
+@pytest.fixture()
+def runtime(fake):
+    fake.fake_set_device(0)
+    fake.fake_fail_launches(0, 0)
+    yield fake
+    fake.fake_fail_launches(0, 0)
+    fake.fake_set_device(0)
+
+
+def at(plane):
+    return BUF.ctypes.data + 4 * plane * PLANE
+
+
+def frame(s):
+    s.denoise(at(0), at(3), at(8), variance=at(5), features=at(16))
+
+
+PAPER = [dict(), dict(state_precision=W.WRLS_STATE_BF16), dict(state_precision=W.WRLS_STATE_F16), dict(blend_mode=1)]
+EXTENDED = [dict(n_gbuf=4, n_features=4), dict(n_gbuf=2, n_features=2), dict(weight_mode=2), dict(reproj_filter=1),
+            dict(n_gbuf=4, n_features=4, blend_mode=1), dict(n_gbuf=4, n_features=4, feature_mode=1)]
+
+
+@pytest.mark.parametrize("kw", PAPER + EXTENDED, ids=str)
+def test_every_device_of_a_process_is_set_up(runtime, kw):
+    """A kernel's opt-in to large shared memory belongs to a device: streams on a second one work too,
+    through per-frame, sequence and batched calls and with every blend configuration."""
+    for dev in (0, 1, 0):
+        assert runtime.fake_set_device(dev) == 0
+        p = W.wrls_params_default(**kw)
+        s = W.Stream(WIDTH, HEIGHT, p)
+        frame(s)
+        W.wrls_denoise_sequence(s.handle, [(at(0), at(5), at(16), at(3), at(8 + 4 * (k & 1))) for k in range(4)])
+        if kw in PAPER:
+            b = W.wrls_batch_create(1)
+            W.wrls_batch_tick(b, [(s.handle, at(0), None, None, at(3), at(8))])
+            W.wrls_batch_destroy(b)
+            W.wrls_batch_tick_static([(s.handle, at(0), None, None, at(3), at(8))])
+            for cfg in range(W.BLEND_CONFIGS):
+                if 4 <= cfg <= 7 and p.state_precision != W.WRLS_STATE_F32:
+                    continue
+                W.wrls_stream_set_blend_config(s.handle, cfg)
+                frame(s)
+        s.close()
