@@ -119,7 +119,10 @@ struct KernelSetup {
     if (!occ) {
       e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem_bytes);
-      if (e != cudaSuccess) return e;
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+      }
       if (occ < 1) occ = 1;
       if (keep) per_sm[dev].store(occ, std::memory_order_release);
     }
@@ -138,7 +141,8 @@ inline bool pdl_allowed(cudaStream_t cs) {
   return cap == cudaStreamCaptureStatusNone;
 }
 
-// Launch, with the programmatic-serialisation attribute if `pdl` (kernels that call pdl_wait).
+// Launch, with the programmatic-serialisation attribute if `pdl` (kernels that call pdl_wait). A failure
+// is in the result alone: it is taken off the runtime's last error, which a caller's own check reads next.
 template <class... P, class... A>
 inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t cs, bool pdl, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -151,7 +155,9 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 // Return WRLS_ERR_CUDA with a message from an entry point when a CUDA call fails.

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 
 from paper_2106_08034_gb300 import build as B
+from paper_2106_08034_gb300 import synth
 from paper_2106_08034_gb300 import wrls as W
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -81,3 +82,38 @@ def test_every_device_of_a_process_is_set_up(runtime, kw):
                 W.wrls_stream_set_blend_config(s.handle, cfg)
                 frame(s)
         s.close()
+
+
+def test_a_failed_launch_leaves_no_error_pending(runtime):
+    """The status reports it; the caller's next check of the runtime's last error finds nothing."""
+    s, e = W.Stream(WIDTH, HEIGHT, W.wrls_params_default()), W.Stream(WIDTH, HEIGHT, W.wrls_params_default(**EXTENDED[0]))
+    frame(s)
+    frame(e)
+    samples = np.zeros((1, 5, HEIGHT, WIDTH), np.float32)
+    planes = BUF.reshape(-1, HEIGHT, WIDTH)
+
+    class Array:  # a buffer with the attributes that the binding reads
+        def __init__(self, a):
+            self.shape, self.data_ptr = a.shape, lambda: a.ctypes.data
+    scene = W.vpt_scene_struct(synth.vpt_scene(WIDTH, HEIGHT, t=0, seed=1))
+    io = [(at(0), at(5), at(16), at(3), at(8 + 4 * (k & 1))) for k in range(2)]
+    calls = [lambda: frame(s), lambda: frame(e), lambda: W.wrls_denoise_sequence(s.handle, io),
+             lambda: W.wrls_denoise_sequence(e.handle, io), lambda: s.write_state(at(0)), lambda: s.read_state(at(0)),
+             lambda: W.wrls_reconstruct(Array(samples), Array(planes[:3])),
+             lambda: W.wrls_velocity_from_world(Array(planes[:3]), np.eye(4), Array(planes[3:5])),
+             lambda: W.wrls_render_vpt(scene, Array(samples), Array(planes[:3]))]
+    for call in calls:
+        for ok in range(2):  # the first or the second launch of the call fails
+            runtime.fake_fail_launches(0, 0)
+            call()
+            n = runtime.fake_launches()
+            call()
+            if ok >= runtime.fake_launches() - n:
+                continue
+            runtime.fake_fail_launches(ok, 1)
+            with pytest.raises(W.WrlsError) as err:
+                call()
+            assert err.value.status == W.WRLS_ERR_CUDA
+            assert runtime.fake_last_error() == 0
+    s.close()
+    e.close()
