@@ -291,7 +291,8 @@ wrls_status wrls_stream_set_blend_config(wrls_stream* s, int config);
  * update kernel arms the mbarrier of each tile's state-window copy but does not issue the
  * copy, so the tile's bounded wait runs out (about one second of SM clocks); the kernel then
  * records WRLS_ERR_TIMEOUT in the stream's error word (read by wrls_stream_check) and
- * returns. The frame's output and state are unreliable; the CUDA context stays usable.
+ * returns. On the extended path, whose windows are copied in parts, the last part is withheld, in
+ * the update and in the two-wide blend. The frame's output and state are unreliable; the CUDA context stays usable.
  * WRLS_DEBUG_NO_THIRD_COPY: the sequence entries keep two state copies, as when the
  * allocation of the third fails (the update of frame t+2 then waits for the blend of frame
  * t). Takes effect if set before the stream's first wrls_denoise_sequence or

@@ -41,7 +41,7 @@ struct KParams {
   int blend_mode;
   int feature_mode;
   int init_mode;
-  int debug_withhold_copy;  // test hook: arm the state-window barrier without issuing the copy
+  int debug_withhold_copy;  // test hook: arm the state-window barrier without issuing the (last) copy
   // host-side launch hints: bits 0-7 CTAs per SM of the persistent blends (0 = all that fit), bit 8
   // start beside the tail of the kernel before (pdl_wait)
   int hints;
@@ -214,13 +214,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t phase) {
       : "memory");
   return ok != 0;
 }
-// Wait for the completion of phase `phase`; false if it did not complete in kWaitLimit clocks.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t phase) {
-  const long long t0 = clock64();
+// Wait for the completion of phase `phase`; false if it did not complete within kWaitLimit clocks of t0
+// (waits of one t0 share the limit).
+__device__ __forceinline__ bool mbar_wait_until(uint64_t* bar, uint32_t phase, const long long t0) {
   while (!mbar_try_wait(bar, phase)) {
     if (clock64() - t0 > kWaitLimit) return false;
   }
   return true;
+}
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t phase) {
+  return mbar_wait_until(bar, phase, clock64());
 }
 // Order this thread's generic-proxy shared-memory accesses before later async-proxy (TMA) ones.
 __device__ __forceinline__ void fence_proxy_async() {

@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
     mbar_expect_tx(&bar[1], (uint32_t)L::kNP * kStagePix * 4u);
     tma_load_3d(stage + S::kOffP, &maps.p, X0, Y0, L::kP, &bar[1]);
     mbar_expect_tx(&bar[2], 3u * D * kStagePix * 4u);
-    tma_load_3d(stage + S::kOffB, &maps.beta, X0, Y0, L::kBeta, &bar[2]);
+    if (!kp.debug_withhold_copy) tma_load_3d(stage + S::kOffB, &maps.beta, X0, Y0, L::kBeta, &bar[2]);
   }
   float I[3] = {0.0f, 0.0f, 0.0f}, lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   bool missing = true;
@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
   auto landed = [&](int k) {
     if (mbar_wait_bounded(&bar[k], 0)) return true;
     atomicExch(err, (int)WRLS_ERR_TIMEOUT);
-    for (int m = 0; m < 3; ++m) mbar_wait_bounded(&bar[m], 0);  // the copies may still be in flight
+    const long long t0 = clock64();
+    for (int m = 0; m < 3; ++m) mbar_wait_until(&bar[m], 0, t0);  // the copies may still be in flight
     return false;
   };
   auto at_once = [](int) { return true; };
@@ -557,7 +558,7 @@ __global__ void __launch_bounds__(128)
     mbar_expect_tx(&zbar, 3u * P * 4u);
     tma_load_3d(w + Z * P, &maps.z, bx0 - 4, by0 - 2, L::kZ, &zbar);
     mbar_expect_tx(&bbar, 3u * D * P * 4u);
-    tma_load_3d(w, &maps.beta, bx0 - 4, by0 - 2, 0, &bbar);
+    if (!kp.debug_withhold_copy) tma_load_3d(w, &maps.beta, bx0 - 4, by0 - 2, 0, &bbar);
   }
   // G-buffer entries of the thread's predictors (.x: column 2 tx, .y: column 2 tx + 1)
   const size_t npix = (size_t)W * H;
@@ -576,7 +577,7 @@ __global__ void __launch_bounds__(128)
   __syncthreads();  // the barriers are initialised
   bool ok = mbar_wait_bounded(&zbar, 0);
   const bool inner = bx0 >= 4 && bx0 + 68 <= W && by0 >= 2 && by0 + 10 <= H;
-  if (!inner) ok = mbar_wait_bounded(&bbar, 0) && ok;  // far records overwrite the beta planes too
+  if (!inner) ok = ok && mbar_wait_bounded(&bbar, 0);  // far records overwrite the beta planes too
   if (ok)
     for (int i = threadIdx.x; i < P; i += 128) {
       const int gx = bx0 - 4 + i % SW, gy = by0 - 2 + i / SW;
@@ -591,11 +592,12 @@ __global__ void __launch_bounds__(128)
         w[(Z + 3) * P + i] = 0.0f;
       }
     }
-  ok = mbar_wait_bounded(&bbar, 0) && ok;
+  ok = ok && mbar_wait_bounded(&bbar, 0);
   if (__syncthreads_or(!ok)) {
     if (threadIdx.x == 0) atomicExch(err, (int)WRLS_ERR_TIMEOUT);
-    mbar_wait_bounded(&zbar, 0);  // the copies may still be in flight
-    mbar_wait_bounded(&bbar, 0);
+    const long long t0 = clock64();
+    mbar_wait_until(&zbar, 0, t0);  // the copies may still be in flight
+    mbar_wait_until(&bbar, 0, t0);
     return;
   }
   pdl_next();
