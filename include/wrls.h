@@ -270,11 +270,12 @@ uint64_t wrls_stream_frames(const wrls_stream* s);
  * denoised frame; `out` (device, 3 x H x W) is overwritten and ends up holding the current
  * frame's output. times_ms (optional, WRLS_BLEND_CONFIGS entries) receives the mean time per
  * launch (-1 for a configuration the state format does not offer) and *chosen (optional)
- * the selected configuration. Synchronises the stream. After wrls_stream_create the
- * configuration is, on images of at least 2^17 pixels (and 72 x 20), 9 for the binary32 state and 8
- * for the 16-bit formats, else 2. wrls_batch_tick uses each stream's configuration; wrls_batch_tick_static uses a
- * one-CTA-per-tile configuration of the same tile rows (2 for configurations 8 and 9).
- * Streams on the extended path have
+ * the selected configuration. Synchronises the stream. Without this call or
+ * wrls_stream_set_blend_config each call chooses by the size: on images of at least 2^17 pixels (and
+ * 72 x 20) 9 for the binary32 state and 8 for the 16-bit formats (below 2^19 pixels unless the last wave
+ * of its CTAs would be mostly empty), else 2. wrls_batch_tick uses each stream's configuration;
+ * wrls_batch_tick_static uses a one-CTA-per-tile configuration of the same tile rows (2 for
+ * configurations 8 and 9). Streams on the extended path have
  * one blend configuration: every time is reported as -1 and 0 is chosen, without a launch.
  */
 #define WRLS_BLEND_CONFIGS 10

@@ -300,7 +300,7 @@ static wrls_status enqueue_blend(wrls_stream* s, const KParams& kp, const float*
     ep.kp = kp;
     e = launch_ext_blend(ep, s->dim, next, s->prm.n_gbuf > 0 ? features : nullptr, out, s->err, cs);
   } else {
-    e = launch_blend(kp, s->blend_cfg, next, out, s->err, cs);
+    e = launch_blend(kp, blend_config_of(s, hint_pdl(kp), two_wide_tiles(s)), next, out, s->err, cs);
   }
   if (e != cudaSuccess) {
     set_error("%s: blend kernel launch: %s", who, cudaGetErrorString(e));
@@ -406,6 +406,10 @@ wrls_status wrls_stream_create(int width, int height, const wrls_params* p, wrls
   s->ep.reproj_filter = p->reproj_filter;
   s->ep.wv_k = (float)(3.0 * 1.4426950408889634 / ((double)p->h * (double)p->h));
   cudaGetDevice(&s->device);
+  if (cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess || s->sms < 1) {
+    cudaGetLastError();
+    s->sms = 1;
+  }
   // both state copies, then the device error word
   const size_t scratch = 256;
   cudaError_t e = cudaMalloc(&s->mem, 2 * copy + scratch);
@@ -440,16 +444,6 @@ wrls_status wrls_stream_create(int width, int height, const wrls_params* p, wrls
       delete s;
       return WRLS_ERR_CUDA;
     }
-  }
-  // Default blend configuration, from the measured ranking (us a frame through per-frame calls with
-  // the one-CTA-per-tile 16 x 2 blend (2) / the two-wide one): on images of at least 2^17 pixels the
-  // two-wide packed blend, 64 x 8 tiles (9) for the binary32 state (512x512 25.7 / 23.0, 643x361 24.3 /
-  // 22.1, 1080p 159.5 / 138.8), 64 x 16 tiles (8) for the 16-bit formats (512x512 20.8 / 19.6, 643x361 20.1 /
-  // 19.4, 1080p 133.2 / 130.0); on smaller images 2, where one tile per CTA spreads the work over more
-  // SMs (128x128 8.3 / 8.9, BF16 7.8 / 10.1; at 256x256 the two are within 5 %).
-  if (!ext) {
-    const bool big = (long long)width * height >= (1ll << 17);
-    s->blend_cfg = (big && s->state[0].blend_tma2_ok) ? (p->state_precision == 0 ? 9 : 8) : 2;
   }
   *out = s;
   return WRLS_OK;

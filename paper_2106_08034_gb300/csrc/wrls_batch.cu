@@ -210,7 +210,8 @@ static wrls_status tick_chains(wrls_batch* b, const wrls_frame_io* frames, int n
   for (int i = 0; i < n; ++i) order[i] = i;
   auto px = [&](int i) { return (long long)frames[i].stream->W * frames[i].stream->H; };
   std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return px(a) > px(c); });
-  long long load[wrls_batch::kLanes] = {};
+  long long load[wrls_batch::kLanes] = {}, tiles = 0;
+  for (int i = 0; i < n; ++i) tiles += two_wide_tiles(frames[i].stream);
   for (int j = 0; j < n && e == cudaSuccess; ++j) {
     const int i = order[j];
     int k = 0;
@@ -222,7 +223,7 @@ static wrls_status tick_chains(wrls_batch* b, const wrls_frame_io* frames, int n
     const StateDesc& prev = s->state[s->cur];
     const StateDesc& next = s->state[next_copy(s)];
     e = launch_update(s->kp, prev, next, s->need_reset, frames[i].radiance, frames[i].motion, s->err, ln);
-    if (e == cudaSuccess) e = launch_blend(s->kp, s->blend_cfg, next, frames[i].out, s->err, ln);
+    if (e == cudaSuccess) e = launch_blend(s->kp, blend_config_of(s, false, tiles), next, frames[i].out, s->err, ln);
   }
   for (int k = 0; k < lanes && e == cudaSuccess; ++k) {
     e = cudaEventRecord(b->ev_join[k], b->lane[k]);
@@ -531,7 +532,7 @@ extern "C" wrls_status wrls_batch_tick_static(const wrls_frame_io* frames, int n
   size_t most = 0;
   for (int i = 0; i < n; ++i) {
     const size_t px = (size_t)frames[i].stream->W * frames[i].stream->H;
-    if (px > most) { most = px; cfg = blend_sync_config(frames[i].stream->blend_cfg); }
+    if (px > most) { most = px; cfg = blend_sync_config(blend_config_of(frames[i].stream, false, two_wide_tiles(frames[i].stream))); }
   }
   const int th_b = blend_rows(cfg);
   // The table is built on the stack and passed by value to k_static_fill: the launch copies

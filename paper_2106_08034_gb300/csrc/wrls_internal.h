@@ -212,7 +212,8 @@ struct wrls_stream {
   cudaEvent_t ev_used[kHostSlots] = {};  // slot's inputs no longer read by kernels
   cudaEvent_t ev_done[kHostSlots] = {};  // slot's output written
   cudaEvent_t ev_out[kHostSlots] = {};   // slot's output copied to the host
-  int blend_cfg = 0;            // blend tile configuration
+  int blend_cfg = -1;           // blend tile configuration set by the caller or by autotune (-1: by rule, blend_config_of)
+  int sms = 1;                  // SMs of the device
   // wrls_denoise_sequence: blends on a second CUDA stream, ordered by events
   cudaStream_t side = nullptr;
   cudaEvent_t ev_u = nullptr;          // update of frame t done (side stream waits)
@@ -230,3 +231,31 @@ struct wrls_stream {
 
 // The state copy the next frame writes: the one after `cur` in the rotation.
 inline int next_copy(const wrls_stream* s) { return s->cur + 1 < s->ncopies ? s->cur + 1 : 0; }
+
+// 64 x 16 tiles of a frame's blend (configuration 8).
+inline long long two_wide_tiles(const wrls_stream* s) { return (long long)((s->W + 63) / 64) * ((s->H + 15) / 16); }
+
+// Blend configuration of a call: the one set on the stream, else by rule. `early`: the kernels are
+// launched before the one ahead of them has ended (per-frame calls); `tiles`: two_wide_tiles of all the
+// blends that run side by side (the frames of a tick). Below 2^17 pixels the one-CTA-per-tile 16 x 2 blend (2)
+// spreads the work over more SMs; from 2^17 the two-wide packed blends are the faster ones: with the
+// binary32 state 64 x 8 tiles (9) through every entry, with the 16-bit formats 64 x 16 tiles (8), two CTAs
+// an SM, where their last wave is not mostly empty: from 2^19 pixels always, below when the waves are 3/4
+// full, and through per-frame calls also when one wave takes them all. Measured, us a frame with 2 / the
+// two-wide one, per-frame calls, sequence, tick of 1, tick of 4 (steps of 2 in the tick of 1):
+//   binary32  361x363 20.2 / 17.8, 14.1 / 12.8, 18.6 / 16.6, 13.2 / 10.6; 643x361 25.0 / 22.0, 19.7 / 18.5,
+//             26.8 / 24.8, 21.5 / 16.8; 854x480 37.4 / 34.6, 32.3 / 27.5, 41.1 / 36.7, 34.6 / 27.0
+//   BF16 643x361 (0.83 of a wave)  22.1 / 21.3, 18.3 / 17.1, 24.8 / 24.6, 17.1 / 16.5
+//        400x400 (0.58)            18.7 / 17.7, 13.7 / 15.0, 18.7 / 20.7, 12.2 / 12.1
+//        854x480 (1.38)            31.0 / 33.0, 25.7 / 26.0, 34.9 / 37.0, 27.0 / 25.7
+//        800x600 (1.63)            36.6 / 36.3, 29.9 / 29.7, 39.1 / 39.1, 30.7 / 29.2
+// (FP16 within 2 % of BF16 but in a sequence at 854x480, 25.9 / 27.1, and 800x600, 30.1 / 30.7.)
+inline int blend_config_of(const wrls_stream* s, bool early, long long tiles) {
+  if (s->blend_cfg >= 0) return s->blend_cfg;
+  const long long px = (long long)s->W * s->H;
+  if (px < (1ll << 17) || !s->state[0].blend_tma2_ok) return 2;
+  if (s->prm.state_precision == 0) return 9;
+  if (px >= (1ll << 19)) return 8;
+  const long long wave = 2ll * s->sms, waves = (tiles + wave - 1) / wave;
+  return (early && waves == 1) || 4 * tiles >= 3 * waves * wave ? 8 : 2;
+}

@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <map>
+#include <string>
 #include <utility>
 #include <vector>
 
@@ -18,7 +19,9 @@ constexpr int kDefaultSmem = 48 * 1024;
 int g_device = 0, g_skip = 0, g_fail = 0;  // the next launches to let through, then to fail
 cudaError_t g_last = cudaSuccess;
 std::map<std::pair<int, const void*>, int> g_smem;  // (device, kernel) -> opted-in bytes
-int g_launches = 0;
+struct Launch { std::string kernel; int early; };  // early: with programmatic serialisation
+std::vector<Launch> g_launches;
+std::map<const void*, std::string> g_names;
 struct Call { dim3 grid, block; size_t smem; void* stream; };
 std::vector<Call> g_calls;
 
@@ -26,7 +29,7 @@ cudaError_t ret(cudaError_t e) {
   if (e != cudaSuccess) g_last = e;
   return e;
 }
-cudaError_t launch(const void* f, size_t smem) {
+cudaError_t launch(const void* f, size_t smem, int early) {
   if (g_skip > 0) {
     --g_skip;
   } else if (g_fail > 0) {
@@ -35,7 +38,7 @@ cudaError_t launch(const void* f, size_t smem) {
   }
   auto it = g_smem.find({g_device, f});
   if ((long long)smem > (it == g_smem.end() ? kDefaultSmem : it->second)) return ret(cudaErrorInvalidValue);
-  ++g_launches;
+  g_launches.push_back({g_names[f], early});
   return cudaSuccess;
 }
 CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
@@ -46,7 +49,9 @@ CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuui
 
 // ---- the test's side
 EXPORT void fake_fail_launches(int skip, int n) { g_skip = skip; g_fail = n; }
-EXPORT int fake_launches() { return g_launches; }
+EXPORT int fake_launches() { return (int)g_launches.size(); }
+EXPORT const char* fake_launch_kernel(int i) { return g_launches[i].kernel.c_str(); }
+EXPORT int fake_launch_early(int i) { return g_launches[i].early; }
 EXPORT int fake_last_error() { return (int)g_last; }
 EXPORT int fake_set_device(int d) { return cudaSetDevice(d); }
 
@@ -55,7 +60,9 @@ EXPORT void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 EXPORT void __cudaRegisterFatBinaryEnd(void**) {}
 EXPORT void __cudaUnregisterFatBinary(void**) {}
 EXPORT void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
-EXPORT void __cudaRegisterFunction(void**, const char*, char*, const char*, int, uint3*, uint3*, dim3*, dim3*, int*) {}
+EXPORT void __cudaRegisterFunction(void**, const char* f, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) {
+  g_names[f] = name;
+}
 EXPORT unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, struct CUstream_st* s) {
   g_calls.push_back({g, b, smem, s});
   return 0;
@@ -71,10 +78,14 @@ EXPORT cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* smem, vo
 }
 EXPORT cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) { *k = (cudaKernel_t)f; return cudaSuccess; }
 EXPORT cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t smem, cudaStream_t) {
-  return launch((const void*)k, smem);
+  return launch((const void*)k, smem, 0);
 }
 EXPORT cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
-  return launch(f, c->dynamicSmemBytes);
+  int early = 0;
+  for (unsigned i = 0; i < c->numAttrs; ++i)
+    early |= c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization &&
+             c->attrs[i].val.programmaticStreamSerializationAllowed;
+  return launch(f, c->dynamicSmemBytes, early);
 }
 EXPORT cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) g_smem[{g_device, f}] = v;

@@ -1,4 +1,5 @@
 """Host side of the launches, followed with a stand-in CUDA runtime of two devices (no GPU needed)."""
+import ctypes
 import glob
 import os
 import subprocess
@@ -34,6 +35,7 @@ def fake(tmp_path_factory):
     saved = W._lib, W.LIB_PATH
     W._lib, W.LIB_PATH = None, so
     try:
+        W.lib().fake_launch_kernel.restype = ctypes.c_char_p
         yield W.lib()
     finally:
         W._lib, W.LIB_PATH = saved
@@ -117,3 +119,55 @@ def test_a_failed_launch_leaves_no_error_pending(runtime):
             assert runtime.fake_last_error() == 0
     s.close()
     e.close()
+
+
+def launched(runtime, call):
+    """[(kernel, launched early)] of a call."""
+    n = runtime.fake_launches()
+    call()
+    return [(runtime.fake_launch_kernel(k).decode(), runtime.fake_launch_early(k)) for k in range(n, runtime.fake_launches())]
+
+
+def blends(runtime, call):
+    """The blend configurations of a call: 2 (one CTA a tile), 8 or 9 (two-wide)."""
+    out = set()
+    for name, _ in launched(runtime, call):
+        if "blend" in name:
+            out.add(9 if "k_blend_tma2ILi8E" in name else 8 if "k_blend_tma2hILi16E" in name else
+                    2 if "k_blendI" in name and "ELi16ELi2E" in name else name)
+    return out
+
+
+# two-wide configuration (9, 8) or 2 by default, through per-frame calls, sequences, a tick of one stream and
+# a tick of four: by the waves of 64 x 16 tiles on 2 x 152 CTAs for the 16-bit formats
+@pytest.mark.parametrize("width,height,f32,half", [
+    (256, 256, (2, 2, 2, 2), (2, 2, 2, 2)),
+    (361, 363, (2, 2, 2, 2), (2, 2, 2, 2)),      # 29 pixels short of 2^17
+    (512, 256, (9, 9, 9, 9), (8, 2, 2, 8)),      # 128 tiles: 0.42 of a wave; four streams 1.68 waves
+    (400, 400, (9, 9, 9, 9), (8, 2, 2, 8)),      # 175
+    (643, 361, (9, 9, 9, 9), (8, 8, 8, 8)),      # 253: 0.83
+    (608, 608, (9, 9, 9, 9), (2, 2, 2, 8)),      # 380: 1.25 waves, 5 waves of four streams
+    (854, 480, (9, 9, 9, 9), (2, 2, 2, 8)),      # 420: 1.38 waves
+    (800, 600, (9, 9, 9, 9), (8, 8, 8, 8)),      # 494: 1.63
+    (1024, 512, (9, 9, 9, 9), (8, 8, 8, 8)),     # 2^19 pixels
+    (16384, 8, (2, 2, 2, 2), (2, 2, 2, 2)),      # lower than a window
+])
+def test_default_blend_of_each_entry(runtime, width, height, f32, half):
+    plane = width * height
+    buf = np.zeros(40 * plane, np.float32)
+
+    def at(p):
+        return buf.ctypes.data + 4 * p * plane
+    for prec, want in ((W.WRLS_STATE_F32, f32), (W.WRLS_STATE_BF16, half), (W.WRLS_STATE_F16, half)):
+        ss = [W.Stream(width, height, W.wrls_params_default(state_precision=prec)) for _ in range(4)]
+        s, b = ss[0], W.wrls_batch_create(4)
+        io = [(at(0), None, None, at(3), at(5 + 3 * k)) for k in range(2)]
+        tick = [(x.handle, at(0), None, None, at(3), at(5 + 3 * k)) for k, x in enumerate(ss)]
+        calls = (lambda: s.denoise(at(0), at(3), at(5)), lambda: W.wrls_denoise_sequence(s.handle, io),
+                 lambda: W.wrls_batch_tick(b, tick[:1]), lambda: W.wrls_batch_tick(b, tick))
+        assert [blends(runtime, c) for c in calls] == [{w} for w in want]
+        W.wrls_stream_set_blend_config(s.handle, 2)  # a configuration that was set holds for every entry
+        assert [blends(runtime, c) for c in calls[:3]] == [{2}] * 3
+        W.wrls_batch_destroy(b)
+        for x in ss:
+            x.close()
