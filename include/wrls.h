@@ -258,8 +258,8 @@ uint64_t wrls_stream_frames(const wrls_stream* s);
 /*
  * Autotuner of the blend kernel's tile shape (not in the paper): times every blend tile
  * configuration on the
- * stream's current state, `reps` launches each (>= 1), on the stream's CUDA stream, and
- * keeps the fastest for later frames. Configurations (output tile rows x output rows per
+ * stream's current state, `reps` launches each (>= 1), on the stream's CUDA stream, launched as
+ * wrls_denoise_frame launches it, and keeps the fastest for later frames. Configurations (output tile rows x output rows per
  * thread): 0: 16x4, 1: 8x4, 2: 16x2, 3: 32x4 with one CTA per tile; 4: 16x2, 5: 16x2,
  * 6: 8x2, 7: 16x4 with persistent CTAs whose windows are filled by TMA bulk tensor copies,
  * double-buffered (4, 6: the next window arrives while the current one is blended) or single

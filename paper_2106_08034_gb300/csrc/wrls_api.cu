@@ -841,6 +841,8 @@ wrls_status wrls_stream_autotune(wrls_stream* s, float* out, int reps, float* ti
     set_error("wrls_stream_autotune: event");
     return WRLS_ERR_CUDA;
   }
+  KParams kp = s->kp;  // launched as per-frame calls launch them
+  if (pdl_allowed(s->cs)) kp.hints |= kHintPdl;
   int best = 0;
   float best_ms = 0.0f;
   cudaError_t e = cudaSuccess;
@@ -849,9 +851,9 @@ wrls_status wrls_stream_autotune(wrls_stream* s, float* out, int reps, float* ti
       if (times_ms) times_ms[c] = -1.0f;
       continue;
     }
-    e = launch_blend(s->kp, c, cur, out, s->err, s->cs);  // warm-up (and first-use setup)
+    e = launch_blend(kp, c, cur, out, s->err, s->cs);  // warm-up (and first-use setup)
     if (e == cudaSuccess) e = cudaEventRecord(e0, s->cs);
-    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_blend(s->kp, c, cur, out, s->err, s->cs);
+    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_blend(kp, c, cur, out, s->err, s->cs);
     if (e == cudaSuccess) e = cudaEventRecord(e1, s->cs);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.0f;
@@ -860,7 +862,7 @@ wrls_status wrls_stream_autotune(wrls_stream* s, float* out, int reps, float* ti
     if (times_ms) times_ms[c] = ms;
     if (c == 0 || ms < best_ms) { best = c; best_ms = ms; }
   }
-  if (e == cudaSuccess) e = launch_blend(s->kp, best, cur, out, s->err, s->cs);
+  if (e == cudaSuccess) e = launch_blend(kp, best, cur, out, s->err, s->cs);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->cs);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

@@ -171,3 +171,12 @@ def test_default_blend_of_each_entry(runtime, width, height, f32, half):
         W.wrls_batch_destroy(b)
         for x in ss:
             x.close()
+
+
+def test_autotune_times_what_frames_run(runtime):
+    """The blend of a per-frame call is launched early; so are the launches that autotune compares."""
+    s = W.Stream(WIDTH, HEIGHT, W.wrls_params_default())
+    assert all(early for _, early in launched(runtime, lambda: frame(s)))
+    log = launched(runtime, lambda: W.wrls_stream_autotune(s.handle, at(8), 3))
+    assert len(log) == 1 + W.BLEND_CONFIGS * 4 and all(early for _, early in log)
+    s.close()
