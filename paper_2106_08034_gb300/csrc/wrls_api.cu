@@ -257,6 +257,18 @@ static wrls_status check_frame(const wrls_stream* s, const float* radiance, cons
   return WRLS_OK;
 }
 
+// Whether the kernels of a frame let the next one be set up only as their CTAs end (pdl_next). With
+// more update tiles than half the SMs and up to four for each, the CTAs of a frame are resident together
+// and share SMs: set up early, the next kernel's are placed where the running ones are fewest, two or
+// three on one SM and none on another. Us a frame, per-frame calls, early / held: binary32 200x150 9.7 / 9.3, 256x256
+// 12.8 / 10.4, 361x363 20.0 / 14.2; BF16 14.5 / 9.3, 15.9 / 9.6, 18.3 / 13.1 (without early launch of either
+// kernel 13.3, 13.3, 17.7); d = 8 256x256 20.0 / 16.6. With fewer tiles every CTA finds an SM of its own
+// (128x128 8.5 / 8.7), with more there are several waves (16-bit 400x400 17.7 / 18.0, 1280x720 57.8 / 58.6).
+static bool hold_next(const wrls_stream* s) {
+  const int tiles = ((s->W + 31) / 32) * ((s->H + 7) / 8);
+  return tiles > s->sms / 2 && tiles <= 4 * s->sms;
+}
+
 // The timing events of the next frame (NULL when timing is off).
 static wrls_status timing_slot(wrls_stream* s, cudaEvent_t** ev) {
   *ev = nullptr;
@@ -467,7 +479,7 @@ wrls_status wrls_denoise_frame(wrls_stream* s, const float* radiance, const floa
   if (ev) WRLS_CHECK_CUDA(cudaEventRecord(ev[0], s->cs), "wrls_denoise_frame: event record");
   KParams kp = s->kp;
   // each kernel is set up while the one before finishes (not under stream capture)
-  if (pdl_allowed(s->cs)) kp.hints |= kHintPdl;
+  if (pdl_allowed(s->cs)) kp.hints |= kHintPdl | (hold_next(s) ? kHintHold : 0);
   st = enqueue_update(s, kp, radiance, variance, features, motion, "wrls_denoise_frame");
   if (st != WRLS_OK) return st;
   if (ev) {

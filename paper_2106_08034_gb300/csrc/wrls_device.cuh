@@ -43,11 +43,12 @@ struct KParams {
   int init_mode;
   int debug_withhold_copy;  // test hook: arm the state-window barrier without issuing the (last) copy
   // host-side launch hints: bits 0-7 CTAs per SM of the persistent blends (0 = all that fit), bit 8
-  // start beside the tail of the kernel before (pdl_wait)
+  // start beside the tail of the kernel before (pdl_wait), bit 9 do not let the next one start ahead of
+  // this kernel's end (pdl_next)
   int hints;
 };
 
-constexpr int kHintPdl = 1 << 8;
+constexpr int kHintPdl = 1 << 8, kHintHold = 1 << 9;
 __host__ __device__ inline int hint_ctas(const KParams& kp) { return kp.hints & 0xff; }
 __host__ __device__ inline bool hint_pdl(const KParams& kp) { return (kp.hints & kHintPdl) != 0; }
 
@@ -82,8 +83,13 @@ __device__ __forceinline__ float blend_rk(float z0, float z1, float z2, float ep
 // kernels, waiting CTAs of the kernels after took slots early and were placed unevenly (256x256
 // 16.4 -> 20.8 us a frame, 1080p 144 -> 149). Per-frame calls, us a frame: 128x128 12.3 -> 7.7, 643x361
 // 28.7 -> 22.1 (with the two-wide blend), 1280x720 72.1 -> 67.3, 1080p 142.4 -> 135.9, FP16 1440p 214.6 ->
-// 208.6.
+// 208.6. A kernel that does not call it lets the next one be set up as its CTAs end, which is the better
+// place where all CTAs of both kernels are resident at once but share SMs: placed beside running CTAs,
+// those of the next kernel crowd the SMs with fewer of them (pdl_next(kp), kHintHold: see hold_next).
 __device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next(const KParams& kp) {
+  if (!(kp.hints & kHintHold)) pdl_next();
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Loads of global memory in the kernels that call pdl_wait(). What they read (state planes, frame

@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH, ExtStage<D, F>::kMinCtas)
     lo_x = min(lo_x, r.x); hi_x = max(hi_x, r.y);
     lo_y = min(lo_y, r.z); hi_y = max(hi_y, r.w);
   }
-  pdl_next();
+  pdl_next(kp);
   const int more = nearest ? 0 : 1;
   const int X0 = lo_x & ~3, Y0 = lo_y;  // TMA box origin: 16-byte aligned column
   const bool fits = stage_ok && hi_x >= 0 && min(hi_x + more, W - 1) - X0 < kStageW && min(hi_y + more, H - 1) - Y0 < kStageH;
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(kExtTW * kExtTH / kExtBlendRows)
     }
   }
   __syncthreads();
-  pdl_next();
+  pdl_next(kp);
   const int x = bx0 + threadIdx.x;
   const int ty0 = threadIdx.y * kExtBlendRows;  // first of the thread's two rows in the tile
   const size_t npix = (size_t)W * H;
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(128)
     mbar_wait_until(&bbar, 0, t0);
     return;
   }
-  pdl_next();
+  pdl_next(kp);
   float2 zi[2][3], ri[2], den[2], acc[2][3];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {

@@ -135,7 +135,7 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* 
     return false;
   }
   if (fits) phase ^= 1u;
-  pdl_next();
+  pdl_next(kp);
   if (!inside) return true;
 
   float I[3] = {sm.rad[0][ty + 1][tx + 1], sm.rad[1][ty + 1][tx + 1], sm.rad[2][ty + 1][tx + 1]};
@@ -270,7 +270,7 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, u
     sm.rad[2][ly][lx] = v.b;
   }
   __syncthreads();
-  pdl_next();
+  pdl_next(kp);
   const int lx0 = tx, ly0 = ty, lx1 = tx, ly1 = ty + kPairY;  // window position - 1
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -506,7 +506,7 @@ __device__ __forceinline__ void blend_tile(float4* __restrict__ smem, const KPar
   __syncthreads();
   blend_fill<SV, TH, kTW * TH / R>(sb, szr, kp, W, H, cur, bx0, by0);
   __syncthreads();
-  pdl_next();
+  pdl_next(kp);
   blend_compute<TH, R, MODE>(sb, szr, kp, W, H, out, bx0, by0);
 }
 

@@ -19,9 +19,10 @@ constexpr int kDefaultSmem = 48 * 1024;
 int g_device = 0, g_skip = 0, g_fail = 0;  // the next launches to let through, then to fail
 cudaError_t g_last = cudaSuccess;
 std::map<std::pair<int, const void*>, int> g_smem;  // (device, kernel) -> opted-in bytes
-struct Launch { std::string kernel; int early; };  // early: with programmatic serialisation
+struct Launch { std::string kernel; int early, watched; };  // early: with programmatic serialisation
 std::vector<Launch> g_launches;
 std::map<const void*, std::string> g_names;
+int g_watch = -1;  // byte offset of an int in the first argument of the kernels, kept with each launch
 struct Call { dim3 grid, block; size_t smem; void* stream; };
 std::vector<Call> g_calls;
 
@@ -29,7 +30,7 @@ cudaError_t ret(cudaError_t e) {
   if (e != cudaSuccess) g_last = e;
   return e;
 }
-cudaError_t launch(const void* f, size_t smem, int early) {
+cudaError_t launch(const void* f, size_t smem, int early, void** args) {
   if (g_skip > 0) {
     --g_skip;
   } else if (g_fail > 0) {
@@ -38,7 +39,9 @@ cudaError_t launch(const void* f, size_t smem, int early) {
   }
   auto it = g_smem.find({g_device, f});
   if ((long long)smem > (it == g_smem.end() ? kDefaultSmem : it->second)) return ret(cudaErrorInvalidValue);
-  g_launches.push_back({g_names[f], early});
+  int watched = 0;
+  if (g_watch >= 0) memcpy(&watched, (const char*)args[0] + g_watch, sizeof(int));
+  g_launches.push_back({g_names[f], early, watched});
   return cudaSuccess;
 }
 CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
@@ -51,6 +54,8 @@ CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuui
 EXPORT void fake_fail_launches(int skip, int n) { g_skip = skip; g_fail = n; }
 EXPORT int fake_launches() { return (int)g_launches.size(); }
 EXPORT const char* fake_launch_kernel(int i) { return g_launches[i].kernel.c_str(); }
+EXPORT void fake_watch(int offset) { g_watch = offset; }
+EXPORT int fake_watched(int i) { return g_launches[i].watched; }
 EXPORT int fake_launch_early(int i) { return g_launches[i].early; }
 EXPORT int fake_last_error() { return (int)g_last; }
 EXPORT int fake_set_device(int d) { return cudaSetDevice(d); }
@@ -77,15 +82,15 @@ EXPORT cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* smem, vo
   return cudaSuccess;
 }
 EXPORT cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) { *k = (cudaKernel_t)f; return cudaSuccess; }
-EXPORT cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t smem, cudaStream_t) {
-  return launch((const void*)k, smem, 0);
+EXPORT cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t smem, cudaStream_t) {
+  return launch((const void*)k, smem, 0, args);
 }
-EXPORT cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+EXPORT cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
   int early = 0;
   for (unsigned i = 0; i < c->numAttrs; ++i)
     early |= c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization &&
              c->attrs[i].val.programmaticStreamSerializationAllowed;
-  return launch(f, c->dynamicSmemBytes, early);
+  return launch(f, c->dynamicSmemBytes, early, args);
 }
 EXPORT cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) g_smem[{g_device, f}] = v;

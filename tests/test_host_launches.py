@@ -2,6 +2,7 @@
 import ctypes
 import glob
 import os
+import re
 import subprocess
 
 import numpy as np
@@ -179,4 +180,43 @@ def test_autotune_times_what_frames_run(runtime):
     assert all(early for _, early in launched(runtime, lambda: frame(s)))
     log = launched(runtime, lambda: W.wrls_stream_autotune(s.handle, at(8), 3))
     assert len(log) == 1 + W.BLEND_CONFIGS * 4 and all(early for _, early in log)
+    s.close()
+
+
+def hints_offset():
+    """Byte offset of KParams::hints (all members are 4 bytes wide)."""
+    src = open(os.path.join(B.CSRC, "wrls_device.cuh")).read()
+    body = re.sub(r"//[^\n]*", "", src[src.index("struct KParams {"):])
+    body = body[body.index("{") + 1:body.index("};")]
+    off = 0
+    for name, array in re.findall(r"(?:float|int) (\w+)(\[kMaxTaps\])?;", body):
+        if name == "hints":
+            return off
+        off += 4 * (25 if array else 1)
+    raise AssertionError("KParams::hints not found")
+
+
+# update tiles (32 x 8) against 152 SMs: early where every CTA finds an SM of its own or there are waves
+@pytest.mark.parametrize("width,height,hold", [(128, 128, False), (152, 120, False), (160, 123, True), (200, 150, True),
+                                               (361, 363, True), (512, 304, True), (512, 305, False), (1280, 720, False)])
+@pytest.mark.parametrize("kw", [dict(), dict(state_precision=W.WRLS_STATE_BF16), dict(n_gbuf=4, n_features=4),
+                                dict(reproj_filter=1), dict(blend_mode=1)], ids=str)
+def test_frames_resident_at_once_hold_the_next_kernel(runtime, width, height, hold, kw):
+    """The kernels of a per-frame call let the next one in early except on images whose CTAs share SMs
+    and are all resident; sequences launch plainly, without either hint."""
+    plane = width * height
+    buf = np.zeros(32 * plane, np.float32)
+
+    def at(p):
+        return buf.ctypes.data + 4 * p * plane
+    s = W.Stream(width, height, W.wrls_params_default(**kw))
+    io = [(at(0), at(5), at(16), at(3), at(8 + 4 * k)) for k in range(2)]
+    runtime.fake_watch(hints_offset())
+    n = runtime.fake_launches()
+    s.denoise(at(0), at(3), at(8), variance=at(5), features=at(16))
+    assert [runtime.fake_watched(k) for k in range(n, n + 2)] == [256 + 512 * hold] * 2
+    n = runtime.fake_launches()
+    W.wrls_denoise_sequence(s.handle, io)
+    assert all(runtime.fake_watched(k) < 256 for k in range(n, n + 4))
+    runtime.fake_watch(-1)
     s.close()
