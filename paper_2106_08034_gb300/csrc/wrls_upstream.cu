@@ -94,7 +94,6 @@ __global__ void __launch_bounds__(kRecThreads, 12)
       if (e < 2 * kRecSH) stage(c, s0 + c, e >> 1, kRecTW + (e & 1));
     }
     const bool near = !__syncthreads_or(wide);
-    if (s0 + kRecChunk >= spp) pdl_next();
     for (int c = 0; c < ns; ++c) {
       const float* w0 = &sm[c][0][warp * kRecR * kRecSW + lane];  // window row and column of dy = dx = -1 of pixel 0
       auto filter = [&](auto all) {
@@ -187,8 +186,10 @@ struct Mat4 {
 
 // V pixels a thread: 4 with 128-bit accesses where every plane's rows allow it (W a multiple of 4,
 // 16-byte aligned buffers), else 1. A streaming kernel: 1080p 12.4 -> 10.3 us, 8.0 with the launch set up
-// beside the kernel before (20 B a pixel, 6.1 us at the copy rate). One pixel a thread does not let the
-// next launch in early: its many small CTAs would contend (12.4 -> 18.8 us).
+// beside the kernel before (20 B a pixel, 6.1 us at the copy rate). Neither form lets the next launch in
+// before its CTAs end: on small images the next kernel's would crowd on the SMs that are free first
+// (reconstruction and velocity in turn, 500x400, 4 samples: 21.4 -> 13.0 us), and beside the many CTAs of one
+// pixel a thread they contend (1080p 12.4 -> 18.8 us).
 template <int V>
 __global__ void k_velocity(const Mat4 M, const int W, const int H, const int miss_policy,
                            const float* world, float* __restrict__ mot) {
@@ -209,7 +210,6 @@ __global__ void k_velocity(const Mat4 M, const int W, const int H, const int mis
       p[c][0] = ld_global(world + c * np + j);
     }
   }
-  if (V == 4) pdl_next();
   const float nan = __int_as_float(0x7fc00000);
 #pragma unroll
   for (int k = 0; k < V; ++k) {

@@ -71,3 +71,11 @@ def test_kernels_launched_early_wait_and_promise_nothing(kernel):
         if first >= 0 and lam and first > lam.start() and first < wait:
             first = body.find(touch, body.index("};", lam.start()))
         assert first < 0 or first > wait, (kernel, touch)
+
+
+@pytest.mark.parametrize("kernel", ["k_reconstruct", "k_velocity", "k_render_vpt"])
+def test_input_steps_let_the_next_kernel_in_as_they_end(kernel):
+    """On small images all their CTAs are resident at once; let in earlier, the next kernel's would
+    crowd on the SMs that are free first."""
+    (_, _, _, body), = [k for k in KERNELS if k[1] == kernel]
+    assert "pdl_wait()" in body and "pdl_next" not in body
