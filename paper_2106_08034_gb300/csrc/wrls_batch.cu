@@ -145,13 +145,6 @@ __global__ void __launch_bounds__(kTW * TH / R)
   }
 }
 
-static int sm_count() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms > 0 ? sms : 1;
-}
-
 static int blend_rows(int cfg) {
   switch (cfg) {
     case 1: return 8;

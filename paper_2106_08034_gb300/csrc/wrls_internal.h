@@ -131,6 +131,14 @@ struct KernelSetup {
   }
 };
 
+// SMs of the current device.
+inline int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 0 ? sms : 1;
+}
+
 // Whether a kernel on `cs` may be launched with that attribute: not under stream capture.
 inline bool pdl_allowed(cudaStream_t cs) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

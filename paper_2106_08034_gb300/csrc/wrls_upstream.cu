@@ -14,9 +14,8 @@
 
 namespace wrls {
 
-// Reconstruction tiles: 32 x 8 pixels, two vertically adjacent pixels a thread.
-constexpr int kRecTW = 32, kRecR = 2, kRecTH = 8;
-constexpr int kRecWarps = kRecTH / kRecR, kRecThreads = 32 * kRecWarps;
+// Reconstruction tiles: 32 x 8 pixels.
+constexpr int kRecTW = 32, kRecTH = 8;
 constexpr int kRecSW = kRecTW + 2, kRecSH = kRecTH + 2, kRecSP = kRecSW * kRecSH;
 
 struct ReconArgs {
@@ -26,33 +25,39 @@ struct ReconArgs {
 
 // I~_j = sum_k g(x_k - x_j) g(y_k - y_j) f_k / sum_k g g over the samples of the 3x3 pixels
 // around j. Samples: ((s * 5 + k) * H + y) * W + x, k = r, g, b, ox, oy. One CTA per 32 x 8
-// tile; the 34 x 10 windows of kRecChunk sample indices at a time are staged in shared
+// tile; the 34 x 10 windows of CH sample indices at a time are staged in shared
 // memory (one barrier pair per chunk). A sample with a non-finite colour or offset, or
 // outside the image, is staged with an infinite offset, which no support contains.
-// The kernel is bound by its instructions and by the latency of each staging phase. Each thread
-// filters two vertically adjacent pixels: a staged sample is read once for both (30 shared loads a
-// pixel and sample index instead of 45), the two rows that reach both pixels run as packed
-// pairs, and where all offsets of the chunk lie within radius - 1 of the pixel centre (always, with
-// the default radius) the support needs no test. The terms of a pixel are still added sample by
-// sample, row by row. 1080p, us: 2 samples a pixel with variance 53.8 -> 50.1, without 51.1 -> 41.3, 3
-// samples 71.5 -> 66.8, 16 samples 332 -> 317. (Four rows a thread: 55-63, fewer warps; 4 sample indices at
-// a time: 58.8; 1: 75.)
-constexpr int kRecChunk = 2;
+// The kernel is bound by its instructions and by the latency of each staging phase. With R = 2 each
+// thread filters two vertically adjacent pixels: a staged sample is read once for both (30 shared loads a
+// pixel and sample index instead of 45) and the two rows that reach both pixels run as packed
+// pairs. Where all offsets of the chunk lie within radius - 1 of the pixel centre (always, with
+// the default radius) the support needs no test. The terms of a pixel are added sample by sample, row by
+// row, by the same operations in both forms. 1080p, us, R = 2 with 2 sample indices at a time: 2 samples a
+// pixel with variance 54.1 -> 50.2, without 51.4 -> 41.5, 3 samples 72.0 -> 68.6, 16 samples 333 -> 317. (Four rows a
+// thread: 55-63, fewer warps; 4 sample indices at a time: 58.8; 1: 75.)
+// On small images, whose CTAs are all resident at once, twice the warps and half the phases are
+// worth more: R = 1 with 4 sample indices at a time. With variance, R = 2 / R = 1, us: 128x128 4 samples 8.3 / 4.5, 16
+// samples 29.4 / 13.6; 300x200 4 samples 9.0 / 5.3; 500x400 (800 tiles) 4 samples 12.0 / 11.1; 643x361 (966) without
+// variance 10.9 / 11.1; 1280x720 33.1 / 36.0.
+constexpr int kRecOneChunk = 4;    // sample indices at a time with one pixel a thread
+constexpr int kRecOneBelow = 6;    // tiles an SM below which a thread takes one pixel
 
-template <bool VAR>
-__global__ void __launch_bounds__(kRecThreads, 12)
+template <bool VAR, int R, int CH>
+__global__ void __launch_bounds__(32 * kRecTH / R, 6 * R)
     k_reconstruct(const ReconArgs a, const int W, const int H, const int spp, const float* smp,
                   float* __restrict__ out, float* __restrict__ var) {
-  __shared__ float sm[kRecChunk][5][kRecSP];
+  constexpr int kWarps = kRecTH / R;
+  __shared__ float sm[CH][5][kRecSP];
   const int bx0 = blockIdx.x * kRecTW, by0 = blockIdx.y * kRecTH;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int x = bx0 + lane, y0 = by0 + warp * kRecR;
+  const int x = bx0 + lane, y0 = by0 + warp * R;
   const size_t np = (size_t)W * H;
-  static_assert(kRecR == 2, "a thread's two pixels are the halves of its sums");
+  static_assert(R == 1 || R == 2, "a thread's pixels are the halves of its sums");
   float2 n0 = make_float2(0.0f, 0.0f), n1 = n0, n2 = n0, den = n0;
   // own samples, shifted by the first valid one (k): sums and sum of squares
-  float k0[kRecR] = {}, k1[kRecR] = {}, k2[kRecR] = {}, m0[kRecR] = {}, m1[kRecR] = {}, m2[kRecR] = {}, q[kRecR] = {};
-  int cnt[kRecR] = {};
+  float k0[R] = {}, k1[R] = {}, k2[R] = {}, m0[R] = {}, m1[R] = {}, m2[R] = {}, q[R] = {};
+  int cnt[R] = {};
   // near: every valid offset of the staged samples is within radius - 1, so that the support holds
   // all of the 3x3 neighbours and needs no test (rounding is monotone and radius representable)
   const float margin = a.radius - 1.0f;
@@ -83,30 +88,37 @@ __global__ void __launch_bounds__(kRecThreads, 12)
     sm[c][4][ew] = oy;
   };
   pdl_wait();
-  for (int s0 = 0; s0 < spp; s0 += kRecChunk) {
-    const int ns = min(kRecChunk, spp - s0);
-    for (int c = 0; c < ns; ++c) {  // a warp takes whole rows, the two left-over columns last
-      // (unrolled: the loads of all of a thread's rows are in flight together)
+  for (int s0 = 0; s0 < spp; s0 += CH) {
+    const int ns = min(CH, spp - s0);
+    if (R == 1) {
+      for (int e = threadIdx.x; e < kRecSP * ns; e += 32 * kWarps) {
+        const int c = e / kRecSP, ew = e - c * kRecSP;
+        stage(c, s0 + c, ew / kRecSW, ew % kRecSW);
+      }
+    } else {
+      for (int c = 0; c < ns; ++c) {  // a warp takes whole rows, the two left-over columns last
+        // (unrolled: the loads of all of a thread's rows are in flight together)
 #pragma unroll
-      for (int k = 0; k < (kRecSH + kRecWarps - 1) / kRecWarps; ++k)
-        if (warp + k * kRecWarps < kRecSH) stage(c, s0 + c, warp + k * kRecWarps, lane);
-      const int e = threadIdx.x;
-      if (e < 2 * kRecSH) stage(c, s0 + c, e >> 1, kRecTW + (e & 1));
+        for (int k = 0; k < (kRecSH + kWarps - 1) / kWarps; ++k)
+          if (warp + k * kWarps < kRecSH) stage(c, s0 + c, warp + k * kWarps, lane);
+        const int e = threadIdx.x;
+        if (e < 2 * kRecSH) stage(c, s0 + c, e >> 1, kRecTW + (e & 1));
+      }
     }
     const bool near = !__syncthreads_or(wide);
     for (int c = 0; c < ns; ++c) {
-      const float* w0 = &sm[c][0][warp * kRecR * kRecSW + lane];  // window row and column of dy = dx = -1 of pixel 0
+      const float* w0 = &sm[c][0][warp * R * kRecSW + lane];  // window row and column of dy = dx = -1 of pixel 0
       auto filter = [&](auto all) {
         constexpr bool ALL = decltype(all)::value;
 #pragma unroll
-        for (int wr = 0; wr < kRecR + 2; ++wr)
+        for (int wr = 0; wr < R + 2; ++wr)
 #pragma unroll
           for (int dx = -1; dx <= 1; ++dx) {
             const float* e = w0 + wr * kRecSW + dx + 1;
             const float r = e[0], g = e[kRecSP], b = e[2 * kRecSP], ox = e[3 * kRecSP], oy = e[4 * kRecSP];
             const float ux = (float)dx + ox;
             const float ux2 = ALL || fabsf(ux) <= a.radius ? ux * ux : INFINITY;  // weight 2^-inf = 0
-            if (wr == 1 || wr == 2) {  // both pixels, packed
+            if (R == 2 && (wr == 1 || wr == 2)) {  // both pixels, packed
               const float2 uy = f2add(make_float2(oy, oy), make_float2((float)(wr - 1), (float)(wr - 2)));
               const float2 t = f2mul(f2fma(uy, uy, make_float2(ux2, ux2)), make_float2(-a.k2, -a.k2));
               float2 w = make_float2(ex2_approx(t.x), ex2_approx(t.y));
@@ -116,10 +128,11 @@ __global__ void __launch_bounds__(kRecThreads, 12)
               n2 = f2fma(w, make_float2(b, b), n2);
               den = f2add(den, w);
             } else {
-              const float uy = (wr == 0 ? -1.0f : 1.0f) + oy;
+              const bool lower = R == 2 && wr == 3;  // the last window row reaches the lower pixel alone
+              const float uy = (float)(lower ? 1 : wr - 1) + oy;
               float w = ex2_approx(fmaf(uy, uy, ux2) * -a.k2);
               if (!ALL) w = fabsf(uy) <= a.radius ? w : 0.0f;
-              if (wr == 0) {
+              if (!lower) {
                 n0.x = fmaf(w, r, n0.x);
                 n1.x = fmaf(w, g, n1.x);
                 n2.x = fmaf(w, b, n2.x);
@@ -138,7 +151,7 @@ __global__ void __launch_bounds__(kRecThreads, 12)
       if (VAR) {
         const float* e = w0 + kRecSW + 1;
 #pragma unroll
-        for (int i = 0; i < kRecR; ++i, e += kRecSW) {
+        for (int i = 0; i < R; ++i, e += kRecSW) {
           const float r = e[0], g = e[kRecSP], b = e[2 * kRecSP];
           const bool own = e[3 * kRecSP] < INFINITY;  // own sample is valid (an invalid one adds 0)
           if (cnt[i] == 0) {
@@ -159,7 +172,7 @@ __global__ void __launch_bounds__(kRecThreads, 12)
   }
   if (x >= W) return;
 #pragma unroll
-  for (int i = 0; i < kRecR; ++i) {
+  for (int i = 0; i < R; ++i) {
     if (y0 + i >= H) break;
     const size_t j = (size_t)(y0 + i) * W + x;
     const float d = i ? den.y : den.x;
@@ -173,7 +186,7 @@ __global__ void __launch_bounds__(kRecThreads, 12)
       } else {
         // sum over channels of sum_s (f - mean)^2 = sum u^2 - (sum u)^2 / n, u = f - k
         const float fn = (float)cnt[i];
-        const float ss = q[i] - (m0[i] * m0[i] + m1[i] * m1[i] + m2[i] * m2[i]) / fn;
+        const float ss = q[i] - fmaf(m2[i], m2[i], fmaf(m1[i], m1[i], m0[i] * m0[i])) / fn;
         var[j] = fmaxf(ss, 0.0f) / (3.0f * (fn - 1.0f)) / fn;
       }
     }
@@ -294,8 +307,11 @@ wrls_status wrls_reconstruct(int width, int height, int spp, const float* sample
   a.radius = p->radius;
   const dim3 grid((width + kRecTW - 1) / kRecTW, (height + kRecTH - 1) / kRecTH);
   cudaStream_t cs = (cudaStream_t)cuda_stream;
-  cudaError_t e = launch_kernel(variance ? k_reconstruct<true> : k_reconstruct<false>, grid, kRecThreads, 0, cs, pdl_allowed(cs),
-                                a, width, height, spp, samples, radiance, variance);
+  const bool one = (int)(grid.x * grid.y) < kRecOneBelow * sm_count();  // one pixel a thread (see the kernel)
+  cudaError_t e = launch_kernel(one ? (variance ? k_reconstruct<true, 1, kRecOneChunk> : k_reconstruct<false, 1, kRecOneChunk>)
+                                    : (variance ? k_reconstruct<true, 2, 2> : k_reconstruct<false, 2, 2>),
+                                grid, one ? 32 * kRecTH : 32 * kRecTH / 2, 0, cs, pdl_allowed(cs), a, width, height, spp, samples,
+                                radiance, variance);
   if (e != cudaSuccess) {
     set_error("wrls_reconstruct: launch: %s", cudaGetErrorString(e));
     return WRLS_ERR_CUDA;

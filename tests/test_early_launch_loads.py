@@ -44,7 +44,7 @@ def _kernels():
 
 KERNELS = list(_kernels())
 LAUNCHED_EARLY = sorted({n for src in SOURCES.values()
-                         for n in re.findall(r"launch_kernel\((?:variance \? |vec \? )?(k_\w+)", src)})
+                         for n in re.findall(r"launch_kernel\((?:\w+ \? \(?)*(k_\w+)", src)})
 
 
 def test_the_kernels_are_found():

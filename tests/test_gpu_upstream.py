@@ -173,3 +173,38 @@ def test_reconstruction_with_a_very_wide_filter(sigma, size, radius, far):
     assert np.isfinite(ref).all() and np.isfinite(got).all()
     assert np.abs(got - ref).max() <= (9 * 2 + 8) * 2.0 ** -22  # as in the tile-edge test
     assert np.array_equal(np.isnan(gv), np.isnan(rvar))
+
+
+# from 6 tiles an SM a thread takes two pixels: the same tile edges on images of that size, and the
+# bits of the one-pixel form on a part of it
+@pytest.mark.parametrize("size", [(1025, 225), (1056, 233), (991, 248)])
+@pytest.mark.parametrize("spp,radius,far", [(1, 1.5, False), (2, 1.5, True), (5, 0.6, True)])
+def test_reconstruction_two_pixels_a_thread(size, spp, radius, far):
+    w, h = size
+    gen = torch.Generator().manual_seed(w * 100 + h + spp)
+    smp = torch.rand(spp, 5, h, w, generator=gen)
+    smp[:, 3:] -= 0.5
+    if far:
+        smp[:, 3:][torch.rand(spp, 2, h, w, generator=gen) < 0.1] *= 2.5
+    smp[:, 0][torch.rand(spp, h, w, generator=gen) < 0.1] = float("nan")
+    p = W.wrls_recon_params_default(radius=radius)
+
+    def run(s):
+        d = s.contiguous().cuda()
+        rad, var = torch.empty(3, *s.shape[2:], device="cuda"), torch.empty(*s.shape[2:], device="cuda")
+        W.wrls_reconstruct(d, rad, var, p)
+        only = torch.empty_like(rad)
+        W.wrls_reconstruct(d, only, None, p)
+        assert torch.equal(rad.nan_to_num(nan=-7.0), only.nan_to_num(nan=-7.0))
+        return rad.cpu(), var.cpu()
+    rad, var = run(smp)
+    ref, rvar = O.reconstruct(smp.numpy(), radius=float(np.float32(radius)))
+    got, fin = rad.numpy(), np.isfinite(ref[0])
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert np.abs(got[:, fin] - ref[:, fin]).max(initial=0.0) <= (9 * spp + 8) * 2.0 ** -22
+    assert np.array_equal(np.isnan(var.numpy()), np.isnan(rvar))
+    assert np.abs(var.numpy() - rvar)[np.isfinite(rvar)].max(initial=0.0) <= (spp + 8) * 2.0 ** -22
+    y, x = h - 41, w - 67  # an inner part, and its pixels whose 3x3 neighbours lie in it
+    prad, pvar = run(smp[:, :, y - 50:y, x - 90:x])
+    assert torch.equal(prad[:, 1:-1, 1:-1].nan_to_num(nan=-7.0), rad[:, y - 49:y - 1, x - 89:x - 1].nan_to_num(nan=-7.0))
+    assert torch.equal(pvar[1:-1, 1:-1].nan_to_num(nan=-7.0), var[y - 49:y - 1, x - 89:x - 1].nan_to_num(nan=-7.0))

@@ -59,6 +59,13 @@ def frame(s):
     s.denoise(at(0), at(3), at(8), variance=at(5), features=at(16))
 
 
+class Array:
+    """A buffer with the attributes that the binding reads."""
+
+    def __init__(self, a):
+        self.shape, self.data_ptr = a.shape, lambda: a.ctypes.data
+
+
 PAPER = [dict(), dict(state_precision=W.WRLS_STATE_BF16), dict(state_precision=W.WRLS_STATE_F16), dict(blend_mode=1)]
 EXTENDED = [dict(n_gbuf=4, n_features=4), dict(n_gbuf=2, n_features=2), dict(weight_mode=2), dict(reproj_filter=1),
             dict(n_gbuf=4, n_features=4, blend_mode=1), dict(n_gbuf=4, n_features=4, feature_mode=1)]
@@ -95,9 +102,6 @@ def test_a_failed_launch_leaves_no_error_pending(runtime):
     samples = np.zeros((1, 5, HEIGHT, WIDTH), np.float32)
     planes = BUF.reshape(-1, HEIGHT, WIDTH)
 
-    class Array:  # a buffer with the attributes that the binding reads
-        def __init__(self, a):
-            self.shape, self.data_ptr = a.shape, lambda: a.ctypes.data
     scene = W.vpt_scene_struct(synth.vpt_scene(WIDTH, HEIGHT, t=0, seed=1))
     io = [(at(0), at(5), at(16), at(3), at(8 + 4 * (k & 1))) for k in range(2)]
     calls = [lambda: frame(s), lambda: frame(e), lambda: W.wrls_denoise_sequence(s.handle, io),
@@ -220,3 +224,12 @@ def test_frames_resident_at_once_hold_the_next_kernel(runtime, width, height, ho
     assert all(runtime.fake_watched(k) < 256 for k in range(n, n + 4))
     runtime.fake_watch(-1)
     s.close()
+
+
+@pytest.mark.parametrize("width,height,one", [(64, 64, True), (643, 320, True), (640, 364, False), (1920, 1080, False)])
+def test_reconstruction_takes_one_pixel_a_thread_on_small_images(runtime, width, height, one):
+    """Below 6 tiles an SM (912 of 32 x 8 on 152), with and without variance."""
+    samples, out = np.zeros((2, 5, height, width), np.float32), np.zeros((4, height, width), np.float32)
+    for var in (None, Array(out[3])):
+        (name, early), = launched(runtime, lambda: W.wrls_reconstruct(Array(samples), Array(out[:3]), var))
+        assert early and ("k_reconstructILb%dELi%dE" % (var is not None, 1 if one else 2)) in name
