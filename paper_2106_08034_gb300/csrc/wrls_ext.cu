@@ -16,8 +16,8 @@
 //
 // The update stages a 40 x 10 window of the previous state per 32 x 8 tile by TMA (three boxes: z, P,
 // beta) and takes one pixel a thread; the blend takes two adjacent columns x two rows a thread
-// from a TMA-filled 72 x 12 window (blend_mode 1 and images smaller than the window: one column a
-// thread, plain loads).
+// from a TMA-filled 72 x 12 window (blend_mode 1, images smaller than the window and small images without
+// G-buffer entries: one column a thread, plain loads).
 #include <type_traits>
 
 #include "wrls_internal.h"
@@ -715,7 +715,13 @@ static cudaError_t launch_ext_t(const ExtParams& ep, const StateDesc& prev, cons
 template <int D, bool F>
 static cudaError_t launch_ext_blend_t(const ExtParams& ep, const StateDesc& cur, const float* gbuf, float* out,
                                       int* err, cudaStream_t cs) {
-  if (ep.kp.blend_mode == 0 && cur.ext_tma_ok) {
+  // Without G-buffer entries (d = 4 or 1) the one-column blend is the faster one on images whose CTAs
+  // leave SMs idle: half the outputs a thread, twice the CTAs. Nearest pixel, us a frame through per-frame
+  // calls / sequence, two columns -> one: 128x128 9.7 / 9.3 -> 7.3 / 7.8, 200x150 9.7 / 11.6 -> 8.9 / 10.9, 320x240 (300
+  // tiles) 10.9 / 12.2 -> 10.1 / 12.8; 361x363 (552) 13.7 / 14.1 -> 14.7 / 15.3. With G-buffer entries, whose
+  // window and predictors two columns share, it is slower at every size (128x128, d = 5 11.1 -> 12.8).
+  const bool few = ExtDim<D, F>::kG == 0 && ((cur.W + kExtTW - 1) / kExtTW) * ((cur.H + kExtTH - 1) / kExtTH) <= 2 * sm_count();
+  if (ep.kp.blend_mode == 0 && cur.ext_tma_ok && !few) {
     constexpr int bytes = ext2_smem_bytes<D>();
     static KernelSetup setup;  // per instantiation
     const cudaError_t e = setup(k_blend_ext2<D, F>, 128, bytes);

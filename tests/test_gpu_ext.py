@@ -177,3 +177,11 @@ def test_tile_edges(wh, kw, motion):
             rad[0, :2, :3] = float("nan")
         return rad, mot, var, feat
     run_ext(cpu_frames(spec), w, h, params(**kw), hooks=hooks)
+
+
+# without G-buffer entries the two-column blend starts at more than 2 tiles (32 x 8) an SM
+@pytest.mark.parametrize("wh", [(643, 121), (705, 117)])
+@pytest.mark.parametrize("kw", [dict(reproj_filter=1), dict(weight_mode=2), dict(weight_mode=2, feature_mode=1)], ids=str)
+def test_two_column_blend_without_gbuffer(wh, kw):
+    w, h = wh
+    run_ext(cpu_frames(synth.SceneSpec(w, h, 3, seed=52, motion="orbit", firefly_frac=0.05)), w, h, params(**kw))

@@ -233,3 +233,20 @@ def test_reconstruction_takes_one_pixel_a_thread_on_small_images(runtime, width,
     for var in (None, Array(out[3])):
         (name, early), = launched(runtime, lambda: W.wrls_reconstruct(Array(samples), Array(out[:3]), var))
         assert early and ("k_reconstructILb%dELi%dE" % (var is not None, 1 if one else 2)) in name
+
+
+@pytest.mark.parametrize("width,height,small", [(128, 128, True), (320, 240, True), (320, 241, False), (361, 363, False)])
+@pytest.mark.parametrize("kw,gbuf", [(dict(reproj_filter=1), False), (dict(weight_mode=2), False),
+                                     (dict(weight_mode=2, feature_mode=1), False), (dict(n_gbuf=1, n_features=1), True),
+                                     (dict(n_gbuf=4, n_features=4), True)], ids=str)
+def test_extended_blend_of_small_images(runtime, width, height, small, kw, gbuf):
+    """Without G-buffer entries, up to 2 tiles (32 x 8) an SM: one column a thread; else two columns."""
+    plane = width * height
+    buf = np.zeros(24 * plane, np.float32)
+
+    def at(p):
+        return buf.ctypes.data + 4 * p * plane
+    s = W.Stream(width, height, W.wrls_params_default(**kw))
+    log = launched(runtime, lambda: s.denoise(at(0), at(3), at(8), variance=at(5), features=at(16)))
+    assert "k_update_ext" in log[0][0] and ("k_blend_extI" if small and not gbuf else "k_blend_ext2I") in log[1][0]
+    s.close()
