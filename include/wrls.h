@@ -201,9 +201,10 @@ wrls_status wrls_denoise_sequence_host(wrls_stream* s, const struct wrls_frame_i
 
 /* Not in the paper: CTAs per SM of the persistent blend kernels (blend configurations 4-9)
  * when they overlap an update in wrls_denoise_sequence: fewer leave the update room on every SM. 0 = as many
- * as fit; default 4 (measured, us per frame with 2 / 3 / 4, binary32 state, configuration 9: 720p 61.1 /
- * 58.3 / 57.3, 1080p 131.8 / 127.4 / 125.9, 2160p 523 / 502 / 496; 16-bit state, configuration 8, whose CTAs
- * are twice as large and of which 2 fit: 1080p 129 with 1, 113 with 2).
+ * as fit; default 4 (measured under a moving camera, us per frame with 2 / 3 / 4, binary32 state,
+ * configuration 9: 643x361 20.6 / 19.6 / 19.2, 720p 63.2 / 59.6 / 58.6, 1080p 135.7 / 129.7 / 127.9, 2160p 534 /
+ * 507 / 500; 16-bit state, configuration 8, whose CTAs are twice as large and of which 2 fit: 1080p 129 with 1,
+ * 113 with 2).
  */
 wrls_status wrls_stream_set_overlap(wrls_stream* s, int blend_ctas_per_sm);
 
@@ -293,7 +294,8 @@ wrls_status wrls_stream_set_blend_config(wrls_stream* s, int config);
  * copy, so the tile's bounded wait runs out (about one second of SM clocks); the kernel then
  * records WRLS_ERR_TIMEOUT in the stream's error word (read by wrls_stream_check) and
  * returns. On the extended path, whose windows are copied in parts, the last part is withheld, in
- * the update and in the two-wide blend. The frame's output and state are unreliable; the CUDA context stays usable.
+ * the update and in the blend from TMA-filled windows. The frame's output and state are
+ * unreliable; the CUDA context stays usable.
  * WRLS_DEBUG_NO_THIRD_COPY: the sequence entries keep two state copies, as when the
  * allocation of the third fails (the update of frame t+2 then waits for the blend of frame
  * t). Takes effect if set before the stream's first wrls_denoise_sequence or

@@ -468,19 +468,18 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
   const int tiles_x = (W + TW2 - 1) / TW2;
   const int n_tiles = tiles_x * ((H + TH - 1) / TH);
   // From the last tile to the first: the update has just written the end of the state copy, so the
-  // first windows hit L2, and this kernel ends where the next update begins. 1080p, us a frame
-  // (update + blend, per-frame calls): binary32 137.9 -> 134.5, BF16 126.4 -> 122.2; 2160p BF16 sequence
-  // 438.0 -> 430.7. (FP16 does not gain: 124.8 -> 124.9; counting down gave its kernel slower code, 73
-  // against 67 us, so it flips the index instead.)
+  // first windows hit L2, and this kernel ends where the next update begins. Us a frame, per-frame calls /
+  // sequence, forwards -> so: 720p 67.1 -> 64.1 / 59.4 -> 58.5, 1080p 138.2 -> 133.5 / 129.0 -> 127.7, 2160p 516.1 ->
+  // 509.8 / 502.5 -> 500.4.
   int tile = n_tiles - 1 - (int)blockIdx.x;
   if (tile < 0) return;
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
     mbar_init(&zbar, 1);
   }
-  // the z planes are copied first and on their own barrier: -rk is computed while the beta
-  // planes are in flight. With the prefetch of the next window: 1080p frame 134.5 -> 133.7 us, 720p 65.3
-  // -> 63.9, sequence 125.1 -> 124.6.
+  // the z planes are copied first and on their own barrier: -rk is computed while the beta planes are
+  // in flight. Us a frame, per-frame calls / sequence, waiting for both first -> so: 720p 66.0 -> 65.1 /
+  // 59.3 -> 59.0, 1080p 136.4 -> 134.5 / 129.3 -> 128.3, 2160p 520.0 -> 516.4 / 504.9 -> 501.6.
   auto fill = [&](int t) {
     const int x = (t % tiles_x) * TW2 - 4, y = (t / tiles_x) * TH - 2;
     mbar_expect_tx(&zbar, 3u * P * 4u);
@@ -497,8 +496,8 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
     if (next < 0) {
       pdl_next();
     } else if (threadIdx.x == 0 && hint_pdl(kp)) {
-      // per-frame calls: the next window into L2 (beside an update, whose traffic it delays, this
-      // costs 1 % at 2160p)
+      // per-frame calls: the next window into L2: 720p 65.1 -> 64.5 us a frame, 1080p 134.5 -> 134.1, 2160p
+      // 516.4 -> 511.5 (in a sequence, beside an update, within 0.3 % either way: left out)
       const int x = (next % tiles_x) * TW2 - 4, y = (next / tiles_x) * TH - 2;
       tma_prefetch_3d(mz, x, y, kZ);
       tma_prefetch_3d(mb, x, y, 0);
@@ -614,7 +613,11 @@ __global__ void __launch_bounds__(kTW * TH / R, 65536 / 128 / (kTW * TH / R))
   const CUtensorMap* mz = TH == 16 ? &maps.z16w : &maps.z8w;
   const int tiles_x = (W + TW2 - 1) / TW2;
   const int n_tiles = tiles_x * ((H + TH - 1) / TH);
-  // tiles are walked from the last to the first (k_blend_tma2); FP16 counts up and flips the index
+  // Tiles are walked from the last to the first (k_blend_tma2): us a frame, per-frame calls, forwards ->
+  // backwards, BF16 720p 60.3 -> 57.8, 1080p 128.4 -> 124.1, 1440p 214.2 -> 206.1, 2160p 459.6 -> 447.4; FP16
+  // 60.4 -> 59.3, 129.0 -> 127.3, 213.8 -> 210.4, 460.4 -> 455.5. How the index is counted is a matter of the code
+  // that the compiler makes of it, at every size from 643x361 on: down for BF16 (up 1 % slower, 2160p 454.5
+  // against 449.0), up and flipped for FP16 (down 5 % slower, 1440p 221.7 against 210.4).
   constexpr bool kDown = !std::is_same<T, __half>::value;
   auto pos = [&](int t) { return kDown ? t : n_tiles - 1 - t; };
   int tile = kDown ? n_tiles - 1 - (int)blockIdx.x : (int)blockIdx.x;
