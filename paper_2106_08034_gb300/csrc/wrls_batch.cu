@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kTW * TH / R)
     if (lt < 0) break;
     const FrameWork& w = fw[f];
     const SV cur = make_view<SV>(w.next_base, w.plane_stride, w.pitch);
-    blend_tile<SV, TH, R, MODE>(sm_blend, w.kp, w.W, w.H, cur, w.out, (lt % w.tiles_x) * kTW,
+    blend_tile<SV, TH, R, MODE, true>(sm_blend, w.kp, w.W, w.H, cur, w.out, (lt % w.tiles_x) * kTW,
                                 (lt / w.tiles_x) * TH);
   }
 }

@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kTW * TH / R)
     k_blend(const KParams kp, const int W, const int H, const SV cur, float* __restrict__ out) {
   extern __shared__ float4 sm_blend[];
   pdl_wait();
-  blend_tile<SV, TH, R, MODE>(sm_blend, kp, W, H, cur, out, blockIdx.x * kTW, blockIdx.y * TH);
+  blend_tile<SV, TH, R, MODE, false>(sm_blend, kp, W, H, cur, out, blockIdx.x * kTW, blockIdx.y * TH);
 }
 
 template <class SV>

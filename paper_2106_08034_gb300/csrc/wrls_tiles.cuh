@@ -42,7 +42,10 @@ constexpr int update_smem_bytes() { return (int)sizeof(UpdateSmem<SV>) + 128; } 
 // mbarrier) while all threads stage the radiance tile; the taps are then read from shared
 // memory. Otherwise (large motion spread) the taps are read from global memory.
 // `bar` is the CTA's mbarrier (count 1) and `phase` its current phase. Returns false if the
-// bounded wait for the copy gave up (the error word is set; the caller must return).
+// bounded wait for the copy gave up (the error word is set; the caller must return). PERSIST: the CTA
+// runs several tiles, in a kernel that is launched plainly (the hint of pdl_next is then not read, which
+// for the work-list kernels is a load of the frame's record in every tile).
+template <bool PERSIST>
 __device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* bar, uint32_t& phase, int* err,
                                            const KParams& kp, const int W, const int H,
                                            const bool reset, const bool stage_ok, const StateF32& prev,
@@ -135,7 +138,7 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<StateF32>& sm, uint64_t* 
     return false;
   }
   if (fits) phase ^= 1u;
-  pdl_next(kp);
+  if constexpr (!PERSIST) pdl_next(kp);
   if (!inside) return true;
 
   float I[3] = {sm.rad[0][ty + 1][tx + 1], sm.rad[1][ty + 1][tx + 1], sm.rad[2][ty + 1][tx + 1]};
@@ -188,7 +191,7 @@ __device__ __forceinline__ Rgb load_radiance(const float* rad, size_t npix, int 
 
 // The same tile with a 16-bit state: 128 threads, two pixels each (update_pair). The decode
 // (an exact unpack and P = L L^T at each tap), Eq. 8-14 and the Cholesky factorisation run
-// packed over the two pixels. PERSIST: the CTA runs several tiles.
+// packed over the two pixels.
 template <class SV, bool PERSIST>
 __device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, uint32_t& phase, int* err,
                                            const KParams& kp, const int W, const int H,
@@ -270,7 +273,7 @@ __device__ __forceinline__ bool update_tile(UpdateSmem<SV>& sm, uint64_t* bar, u
     sm.rad[2][ly][lx] = v.b;
   }
   __syncthreads();
-  pdl_next(kp);
+  if constexpr (!PERSIST) pdl_next(kp);
   const int lx0 = tx, ly0 = ty, lx1 = tx, ly1 = ty + kPairY;  // window position - 1
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -361,7 +364,7 @@ constexpr int update_min_ctas() { return SV::kScaled ? 6 : 5; }
 template <class SV, bool PERSIST, class... A>
 __device__ __forceinline__ bool update_any(A&&... a) {
   if constexpr (SV::kScaled) return update_tile<SV, PERSIST>(a...);
-  else return update_tile(a...);
+  else return update_tile<PERSIST>(a...);
 }
 
 // 128-byte aligned view of a dynamic shared-memory buffer.
@@ -496,8 +499,8 @@ __device__ __forceinline__ void blend_compute(const float4* __restrict__ sb,
 }
 
 // Whole blend tile: barrier, fill, barrier, compute (a CTA may run tiles back to back).
-// `smem` is 16-byte aligned and holds BlendGeom<TH>::kSmemBytes.
-template <class SV, int TH, int R, int MODE>
+// `smem` is 16-byte aligned and holds BlendGeom<TH>::kSmemBytes. PERSIST: as in update_tile.
+template <class SV, int TH, int R, int MODE, bool PERSIST>
 __device__ __forceinline__ void blend_tile(float4* __restrict__ smem, const KParams& kp, const int W,
                                            const int H, const SV& cur, float* __restrict__ out,
                                            const int bx0, const int by0) {
@@ -506,7 +509,7 @@ __device__ __forceinline__ void blend_tile(float4* __restrict__ smem, const KPar
   __syncthreads();
   blend_fill<SV, TH, kTW * TH / R>(sb, szr, kp, W, H, cur, bx0, by0);
   __syncthreads();
-  pdl_next(kp);
+  if constexpr (!PERSIST) pdl_next(kp);
   blend_compute<TH, R, MODE>(sb, szr, kp, W, H, out, bx0, by0);
 }
 

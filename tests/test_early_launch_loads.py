@@ -79,3 +79,12 @@ def test_input_steps_let_the_next_kernel_in_as_they_end(kernel):
     crowd on the SMs that are free first."""
     (_, _, _, body), = [k for k in KERNELS if k[1] == kernel]
     assert "pdl_wait()" in body and "pdl_next" not in body
+
+
+def test_work_list_kernels_are_launched_plainly_and_read_no_hint():
+    """Their parameters lie in global memory: the hint of pdl_next would be a load in every tile."""
+    src = SOURCES["wrls_batch.cu"]
+    assert "launch_kernel(" not in src and "pdl_" not in src
+    assert re.findall(r"(?:update_any|blend_tile)<([^>]*)>", src) == ["SV, true", "SV, TH, R, MODE, true"]
+    assert len(re.findall(r"if constexpr \(!PERSIST\) pdl_next\(kp\);", SOURCES["wrls_tiles.cuh"])) == 3
+    assert len(re.findall(r"\bpdl_next\(", SOURCES["wrls_tiles.cuh"])) == 3
